@@ -204,7 +204,7 @@ size_t tt_workspace_bytes_for(const tt_batch* batch, int32_t V_d, int32_t V_t,
  * then (i, j-1). Writes path/path_len/cost/map/status; map[j] is the largest
  * draft index on the path in column j. Uses batch ids (not cols). Needs no
  * workspace. The on-chip tile of a pair takes one byte per band cell (at most
- * about 145 KB of shared memory at max_k = TT_MAX_K, max_m = TT_MAX_M with no
+ * about 175 KB of shared memory at max_k = TT_MAX_K, max_m = TT_MAX_M with no
  * band), so every allowed size fits; TT_ERR_UNSUPPORTED would report one that
  * did not. */
 tt_status tt_align(const tt_batch* batch, const tt_vocab* vd, const tt_vocab* vt,

@@ -298,15 +298,6 @@ void attach_kept(DecideArgs& d, const Workspace& ws) {
   d.um_t = ws.um_t;
 }
 
-// Share of the target rows the step's row pass streams before it waits for
-// the alignment (in eighths): half, or seven eighths when the batch holds so
-// many draft tokens (B x max_k of 32768 and more, each a row of the DTW tile)
-// that the alignment outlasts half of the target rows; the rest is drawn
-// dynamically after the wait.
-int pre_wait_eighths(const tt_batch* b) {
-  return int64_t(b->B) * b->max_k >= 32768 ? 7 : 4;
-}
-
 void record(const tt_params* p, int i, cudaStream_t s) {
   if (p->events && p->events[i]) cudaEventRecord(static_cast<cudaEvent_t>(p->events[i]), s);
 }
@@ -326,17 +317,9 @@ tt_status fill_align_args(const tt_batch* bt, const tt_vocab* vd, const tt_vocab
   a.target_ids = bt->target_ids;
   a.vd = *vd;
   a.vt = *vt;
-  a.tile_w = align_tile_width(bt->max_k, bt->max_m, prm->window);
-  a.smem_per_warp = align_smem_per_warp(bt->max_k, bt->max_m, a.tile_w);
-  if (a.smem_per_warp > size_t(kAlignSmemMax)) return TT_ERR_UNSUPPORTED;
-  // pairs spread over the SMs (one warp each while the batch is small), at
-  // most kAlignWarpsMax warps and 96 KB per CTA; before the row pass,
-  // launch_align caps the grid at one CTA per SM, whose warps then loop over
-  // the pairs
-  int wpb = int(size_t(96 * 1024) / a.smem_per_warp);
-  const int spread = (bt->B + sm_count_current() - 1) / sm_count_current();
-  wpb = std::min(wpb, std::min(kAlignWarpsMax, spread));
-  a.warps_per_block = wpb < 1 ? 1 : wpb;
+  a.tile_blocks = align_tile_blocks(bt->max_k, bt->max_m, prm->window);
+  a.smem_per_pair = align_smem_per_pair(bt->max_k, bt->max_m, a.tile_blocks);
+  if (a.smem_per_pair > size_t(kAlignSmemMax)) return TT_ERR_UNSUPPORTED;
   return TT_OK;
 }
 
@@ -727,7 +710,7 @@ tt_status tt_step(const tt_batch* batch, const tt_vocab* vd, const tt_vocab* vt,
   r.err = ws.err;
   r.epoch = next_epoch();
   r.work = ws.work;       // zeroed by the alignment kernel
-  r.pre_eighths = pre_wait_eighths(batch);
+  r.pre_eighths = 4;
   r.excl_late = ws.excl;  // written by the alignment kernel
   // programmatic dependent launch: target rows stream while the alignment runs
   // (unless stage events sit between the kernels)

@@ -33,8 +33,9 @@ struct AlignArgs {
   const int32_t* target_cols;  // scored column of each target position
   int32_t* excl;               // [n_target + B] written: scored column of each target row
                                // (-1 for the bonus row), may be NULL
-  int warps_per_block, tile_w;
-  size_t smem_per_warp;
+  int tile_blocks;     // 16-byte blocks of a pair's cost tile
+  size_t smem_per_pair;
+  int pairs_per_block; // (set by launch_align)
 };
 
 // One family of logits rows seen by the row pass.
@@ -180,8 +181,8 @@ struct PrepArgs {
   unsigned long long* work;  // row-pass work counter to zero (may be NULL)
 };
 
-size_t align_smem_per_warp(int max_k, int max_m, int tile_w);
-int align_tile_width(int max_k, int max_m, int window);
+size_t align_smem_per_pair(int max_k, int max_m, int tile_blocks);
+int align_tile_blocks(int max_k, int max_m, int window);
 cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream);
 cudaError_t launch_rowpass(const RowPassArgs& args, int dt_d, int dt_t, cudaStream_t stream,
                            int sm_count, bool pdl);
