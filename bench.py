@@ -265,7 +265,7 @@ def step_launches(args) -> int:
     if args.top_k > 0:
         return 5 + pen
     if args.top_p < 1.0:
-        return 6  # the nucleus merge and the exact nucleus kernel
+        return 6  # at most: two nucleus kernels (wide rows take one, in the row pass's place)
     return 3
 
 

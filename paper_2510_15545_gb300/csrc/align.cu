@@ -753,7 +753,8 @@ __global__ void __launch_bounds__(align_threads(WPP), 1024 / align_threads(WPP))
   // before it reads the needed-draft-row flags
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.work && blockIdx.x == 0 && threadIdx.x < kWorkShards)
-    a.work[threadIdx.x * kWorkStride] = 0ull;  // read after this grid ends
+    a.work[threadIdx.x * kWorkStride] = a.work[threadIdx.x * kWorkStride + kNucWork] =
+        0ull;  // read after this grid ends
   if constexpr (WPP == 1) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     char* region = smem_raw + size_t(warp) * a.smem_per_pair;

@@ -39,6 +39,7 @@ cudaError_t ensure_loaded() {
   if ((e = preload_decide()) != cudaSuccess) return e;
   if ((e = preload_filter()) != cudaSuccess) return e;
   if ((e = preload_nucleus()) != cudaSuccess) return e;
+  if ((e = preload_nucleus_rows()) != cudaSuccess) return e;
   if ((e = preload_pen()) != cudaSuccess) return e;
   if ((e = preload_shard()) != cudaSuccess) return e;
   if (dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
@@ -153,10 +154,43 @@ cudaError_t launch_pen_sets(const tt_batch* batch, const RowSet& d, const RowSet
   return launch_pen_prep(a, s);
 }
 
-// A nucleus family's row set: the row pass writes the compensated partials of
-// all its columns, and the nucleus kernel finds each row's kept set from them
-// and the row's logits.
-void attach_nucleus(RowSet& r, bool on) { r.nucleus = on ? 1 : 0; }
+// A nucleus family's row set (see RowSet::nucleus).
+void attach_nucleus(RowSet& r, bool on) { r.nucleus = nucleus_rows(on, r.V); }
+
+// Streams the rows of r: wide nucleus families by the nucleus row kernel, the
+// others by the row pass.
+cudaError_t launch_rows(const RowPassArgs& r, const tt_params* prm, const Workspace& ws, int dt_d,
+                        int dt_t, cudaStream_t s, bool pdl) {
+  RowPassArgs p = r;
+  NucRowArgs n;
+  std::memset(&n, 0, sizeof n);
+  n.d = r.d;
+  n.t = r.t;
+  if (r.d.nucleus == kNucWideRows) {
+    n.rows_d = r.rows_d;
+    p.rows_d = 0;
+    p.d.nucleus = 0;
+  }
+  if (r.t.nucleus == kNucWideRows) {
+    n.rows_t = r.rows_t;
+    p.rows_t = 0;
+    p.t.nucleus = 0;
+  }
+  if (p.rows_d + p.rows_t > 0) {
+    const cudaError_t e = launch_rowpass(p, dt_d, dt_t, s, sm_count_current(), pdl);
+    if (e != cudaSuccess) return e;
+  }
+  n.top_p_d = prm->top_p_draft;
+  n.top_p_t = prm->top_p_target;
+  n.head_d = ws.head_d;
+  n.head_t = ws.head_t;
+  n.um_d = ws.um_d;
+  n.um_t = ws.um_t;
+  n.err = r.err;
+  n.epoch = r.epoch;
+  n.work = r.work;
+  return launch_nucleus_rows(n, dt_d, dt_t, s, sm_count_current(), pdl);
+}
 
 // A family's row set sees its penalty arrays.
 void attach_pen(RowSet& r, bool on, float theta, PenEntry* pen, const int32_t* pbase,
@@ -492,8 +526,7 @@ tt_status tt_transfer(const tt_batch* batch, const int32_t* map, const tt_logits
     d.err = ws.err;
     d.epoch = r.epoch;
     // (the absent family's type is a placeholder: the draft's, one kernel variant)
-    if ((e = launch_rowpass(r, draft->dtype, draft->dtype, s, sm_count_current(), true)) !=
-        cudaSuccess)
+    if ((e = launch_rows(r, prm, ws, draft->dtype, draft->dtype, s, true)) != cudaSuccess)
       return cuda_fail(e);
   }
   if (kd > 0 || nd) {
@@ -587,8 +620,8 @@ tt_status tt_verify(const tt_batch* batch, const float* q_hat, const tt_logits* 
   r.pre_eighths = 4;
   // the first kernel of the chain starts only after the caller's work is
   // complete: it reads the logits before its grid-dependency wait
-  if ((e = launch_rowpass(r, full_q ? draft->dtype : target->dtype, target->dtype, s,
-                          sm_count_current(), full_q)) != cudaSuccess)
+  if ((e = launch_rows(r, prm, ws, full_q ? draft->dtype : target->dtype, target->dtype, s,
+                       full_q)) != cudaSuccess)
     return cuda_fail(e);
 
   DecideArgs d;
@@ -715,8 +748,8 @@ tt_status tt_step(const tt_batch* batch, const tt_vocab* vd, const tt_vocab* vt,
   // programmatic dependent launch: target rows stream while the alignment runs
   // (unless stage events sit between the kernels)
   const bool pdl = prm->events == nullptr;
-  if ((e = launch_rowpass(r, from_logits ? draft->dtype : target->dtype, target->dtype, s,
-                          sm_count_current(), pdl)) != cudaSuccess)
+  if ((e = launch_rows(r, prm, ws, from_logits ? draft->dtype : target->dtype, target->dtype, s,
+                       pdl)) != cudaSuccess)
     return cuda_fail(e);
   record(prm, 2, s);
 

@@ -761,7 +761,8 @@ __global__ void __launch_bounds__(kDecThreads) transfer_kernel(DecideArgs a) {
 __global__ void prep_kernel(PrepArgs a) {
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (a.work && blockIdx.x == 0 && threadIdx.x < kWorkShards)
-    a.work[threadIdx.x * kWorkStride] = 0ull;  // read after this grid ends
+    a.work[threadIdx.x * kWorkStride] = a.work[threadIdx.x * kWorkStride + kNucWork] =
+        0ull;  // read after this grid ends
   if (b >= a.B) return;
   if (a.need && csr_ok(a.draft_off, b, a.n_draft) && csr_ok(a.target_off, b, a.n_target)) {
     const int d0 = a.draft_off[b], k = a.draft_off[b + 1] - d0;

@@ -65,7 +65,7 @@ constexpr int kRetryCands = 3200;      // candidates a second pass may take (of 
 constexpr float kMinBar = 8.f;         // lowest bar of a second pass
 // Rows of at most kWarpRowMax columns: one warp per row (nucleus_warp_kernel),
 // candidates within kWCandDelta log2 units of the maximum, at most kWCap.
-constexpr int kWarpRowMax = 8192;
+constexpr int kWarpRowMax = kNucNarrow;
 constexpr float kWCandDelta = 12.f;
 constexpr int kWCap = 512;
 constexpr int kWBuckets = int(kWCandDelta) * 32 + 32;
@@ -74,7 +74,7 @@ constexpr int kWChunks = kWarpRowMax / kChunk;
 // buckets of the candidates' delta (a little past kCandDelta: the fp32 delta of
 // a candidate may round up to it)
 constexpr int kCandBuckets = int(kCandDelta) * 32 + 32;
-constexpr float kFix = 1099511627776.f;  // 2^40: fixed-point scale of the masses
+constexpr float kFix = kFixScale;  // of the masses
 
 __device__ __forceinline__ float load_dt(const char* row, int dt, int64_t col) {
   return dt == TT_F32 ? load_logit<TT_F32>(row, col) : load_logit<TT_BF16>(row, col);
@@ -297,8 +297,8 @@ __device__ void walk_runs(const Cand* arr, int n, unsigned long long before, dou
 // (a column there weighs at least 2^-kCandDelta of the maximum's mass): those
 // columns are gathered in shared memory, their masses (40-bit fixed point)
 // binned by delta at 1/32 log2 unit, and the bucket where the running mass,
-// largest logits first, reaches top_p of the row's total (from the partials)
-// is walked by value. Every column above zc is a candidate, so the walk over
+// largest logits first, reaches top_p of the row's total Td (the sum of
+// 2^(z * scale - M)) is walked by value. Every column above zc is a candidate, so the walk over
 // the candidates in rank order is the walk over the whole row down to zc, and
 // a cut reached among them is the row's cut. Candidates that overflow the
 // buffer at the first bar are gathered again at a lower one (below). Returns
@@ -307,18 +307,10 @@ __device__ void walk_runs(const Cand* arr, int n, unsigned long long before, dou
 // the crossing bucket holds more than kCross of them. On true, sm.cacc holds
 // the kept masses per chunk.
 // Every thread calls and gets the same result.
-__device__ bool candidate_cut(const Partial* part, NucSmem& sm, const char* row, int dt, int V,
-                              int nvec, int vec, int nch, float M, float scale, float top_p,
-                              float& tau, int& tau_col) {
+__device__ bool candidate_cut(double Td, NucSmem& sm, const char* row, int dt, int V, int nvec,
+                              int vec, int nch, float M, float scale, float top_p, float& tau,
+                              int& tau_col) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // the row's total 2^(z * scale - M), compensated, from the partials
-  F2 T = {0.f, 0.f};
-  for (int c = tid; c < nch; c += kNT) {
-    const Partial q = part[c];
-    if (q.m > -INFINITY) T = f2_add(T, F2{__fmul_rn(q.s, ex2_approx(q.m - M)), 0.f});
-  }
-  T = block_sum_f2(T, sm, lane, warp);
-  const double Td = double(T.hi) + double(T.lo);
   if (!(Td > 0.0) || !isfinite(Td)) return false;
   const double thr = double(top_p) * Td * double(kFix);
   // Candidates: z > zc, zc = (M - bar) / scale. The first pass uses the bar
@@ -678,26 +670,28 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
     unsigned long long tot = lane < nch ? sm.cacc[lane] : 0ull;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    const double Sd = double(tot) / double(kFix);  // kept normaliser relative to 2^M
-    if (lane < nch) um[lane] = float(double(sm.cacc[lane]) / double(kFix) / Sd);
-    if (lane == 0) {
-      const float lse = float((double(M) + log2(Sd)) * 0.6931471805599453);
-      *head = KeptHead{lse, 1, tau, tau_col, M, float(1.0 / Sd)};
-    }
+    const KeptNorm kn = kept_norm(tot, M);
+    if (lane < nch) um[lane] = __ull2float_rn(sm.cacc[lane]) * kn.inv_tot;
+    if (lane == 0) *head = KeptHead{kn.lse, 1, tau, tau_col, M, kn.inv_s};
     __syncwarp();  // shared memory is reused by the warp's next row
   }
 }
 
-// One CTA per nucleus row: every row of a family wider than kWarpRowMax, and
-// the rows of a narrower family that nucleus_warp_kernel left (head n = -1),
-// found 256 rows at a time. Tiles of draft rows, then of target rows,
-// grid-stride.
+// One CTA per nucleus row: the rows that the nucleus row kernel or
+// nucleus_warp_kernel left (head n = -1), found in tiles of at most 256 rows,
+// and every row of a family wider than either takes. Tiles of draft rows, then of target
+// rows, grid-stride.
 __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   extern __shared__ __align__(16) char nsm_raw[];
   NucSmem& sm = *reinterpret_cast<NucSmem*>(nsm_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t rows_d = a.d.nucleus ? a.rows_d : 0, rows_t = a.t.nucleus ? a.rows_t : 0;
-  const int tsz_d = a.d.V <= kWarpRowMax ? kNT : 1, tsz_t = a.t.V <= kWarpRowMax ? kNT : 1;
+  // rows per tile: one when every row is to be done, else a share of the rows
+  auto tile_rows = [&](const RowSet& S, int64_t rows) {
+    const int64_t share = (rows + gridDim.x - 1) / gridDim.x;
+    return S.V <= kNucWideMax ? int(max(int64_t(1), min(int64_t(kNT), share))) : 1;
+  };
+  const int tsz_d = tile_rows(a.d, rows_d), tsz_t = tile_rows(a.t, rows_t);
   const int64_t nt_d = (rows_d + tsz_d - 1) / tsz_d, nt_t = (rows_t + tsz_t - 1) / tsz_t;
   grid_dependency_wait();  // the partials (and the need flags) come from earlier kernels
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -706,20 +700,21 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   const int tsz = tgt ? tsz_t : tsz_d;
   const int64_t r0 = (tgt ? tile - nt_d : tile) * tsz;
   int n_todo = 1;
-  if (tsz > 1) {  // the narrow rows the warp kernel could not settle
+  const bool some = (tgt ? a.t.V : a.d.V) <= kNucWideMax;
+  if (some) {  // the rows an earlier kernel could not settle
     __syncthreads();
     if (tid == 0) sm.n_todo = 0;
     __syncthreads();
     const int64_t rr = r0 + tid;
     const RowSet& SF = tgt ? a.t : a.d;
     const KeptHead* hf = tgt ? a.head_t : a.head_d;
-    if (rr < (tgt ? rows_t : rows_d) && (tgt || !SF.need || SF.need[rr] != 0) && hf[rr].n == -1)
+    if (tid < tsz && rr < (tgt ? rows_t : rows_d) && (tgt || !SF.need || SF.need[rr] != 0) && hf[rr].n == -1)
       sm.todo[atomicAdd(&sm.n_todo, 1)] = tid;
     __syncthreads();
     n_todo = sm.n_todo;
   }
   for (int k = 0; k < n_todo; ++k) {
-    const int64_t r = tsz > 1 ? r0 + sm.todo[k] : r0;
+    const int64_t r = some ? r0 + sm.todo[k] : r0;
     const RowSet& S = tgt ? a.t : a.d;
     if (!tgt && S.need && S.need[r] == 0) continue;
     const int dt = tgt ? a.dt_t : a.dt_d;
@@ -732,15 +727,22 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
     const int vec = dt == TT_F32 ? 4 : 8;  // logits per 16-byte vector
     const int nvec = V / vec;              // whole vectors (rows start on 16 bytes)
 
-    // the row maximum from the partials (nucleus rows' partials hold every column)
+    // the row maximum and total: from the partials (they hold every column), or
+    // as the nucleus row kernel left them
     float M = -INFINITY;
-    for (int c = tid; c < nch; c += kNT) M = fmaxf(M, S.part[r * nch + c].m);
+    F2 T = {0.f, 0.f};
+    if (S.nucleus == kNucWideRows) {
+      const KeptHead h = *head;
+      M = h.M;
+      T = {h.inv_s, h.lse};
+      __syncthreads();  // read by every thread before the header is written again
+    } else {
+      for (int c = tid; c < nch; c += kNT) M = fmaxf(M, S.part[r * nch + c].m);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    __syncthreads();
-    if (lane == 0) sm.wmax[warp] = __float_as_uint(M) ^ (M < 0.f ? 0xffffffffu : 0x80000000u);
-    __syncthreads();
-    {
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      __syncthreads();
+      if (lane == 0) sm.wmax[warp] = __float_as_uint(M) ^ (M < 0.f ? 0xffffffffu : 0x80000000u);
+      __syncthreads();
       unsigned long long best = 0;
 #pragma unroll
       for (int x = 0; x < kNW; ++x) best = max(best, sm.wmax[x]);
@@ -750,6 +752,13 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
     if (!isfinite(M)) {
       if (tid == 0) *head = KeptHead{NAN, 0, NAN, -1, M, 0.f};
       continue;
+    }
+    if (S.nucleus != kNucWideRows) {
+      for (int c = tid; c < nch; c += kNT) {
+        const Partial q = S.part[r * nch + c];
+        if (q.m > -INFINITY) T = f2_add(T, F2{__fmul_rn(q.s, ex2_approx(q.m - M)), 0.f});
+      }
+      T = block_sum_f2(T, sm, lane, warp);
     }
 
     // every column once per pass, 16-byte vectors and the ragged tail
@@ -778,7 +787,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
 
     float tau = -INFINITY;
     int tau_col = 0x7fffffff;  // all kept: every column ranks before (tau, tau_col)
-    const bool settled = candidate_cut(S.part + r * nch, sm, row, dt, V, nvec, vec, nch, M,
+    const bool settled = candidate_cut(double(T.hi) + double(T.lo), sm, row, dt, V, nvec, vec, nch, M,
                                        scale, top_p, tau, tau_col);
     if (!settled) {
     // ------------------------------------- the crossing bucket, level by level
@@ -966,13 +975,9 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
     unsigned long long tot = 0ull;
     for (int c = tid; c < nch; c += kNT) tot += sm.cacc[c];
     tot = block_sum_u64(tot, sm, lane, warp);
-    const double Sd = double(tot) / double(kFix);  // kept normaliser relative to 2^M
-    const float inv_s = float(1.0 / Sd);
-    for (int c = tid; c < nch; c += kNT) um[c] = float(double(sm.cacc[c]) / double(kFix) / Sd);
-    if (tid == 0) {
-      const float lse = float((double(M) + log2(Sd)) * 0.6931471805599453);
-      *head = KeptHead{lse, tot > 0ull ? 1 : 0, tau, tau_col, M, inv_s};
-    }
+    const KeptNorm kn = kept_norm(tot, M);
+    for (int c = tid; c < nch; c += kNT) um[c] = __ull2float_rn(sm.cacc[c]) * kn.inv_tot;
+    if (tid == 0) *head = KeptHead{kn.lse, tot > 0ull ? 1 : 0, tau, tau_col, M, kn.inv_s};
     __syncthreads();  // shared memory is reused by the next row
   }
   }

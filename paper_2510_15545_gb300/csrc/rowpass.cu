@@ -22,6 +22,7 @@
 #include "tt_device.cuh"
 #include "tt_launch.h"
 #include "tt_f2.cuh"
+#include "tt_ring.cuh"
 
 namespace tt {
 
@@ -30,7 +31,6 @@ namespace {
 constexpr int kConsumerWarps = 8;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
 constexpr int kRingBytes = 64 * 1024;  // three CTAs per SM fit
-constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 constexpr int kGrabMinBytes = 16 * 1024;   // smallest draw from the work counter
 constexpr int kGrabMaxBytes = 128 * 1024;  // largest draw
 
@@ -66,59 +66,6 @@ struct Ring {
   static constexpr int kGrabMin = kGrabMinBytes / kStageBytes > 0 ? kGrabMinBytes / kStageBytes : 1;
   static constexpr int kGrabMax = kGrabMaxBytes / kStageBytes;
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Waits for the phase of the given parity to complete; false after limit_ns.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
-                                          const uint64_t& limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t i = 1; i < (1u << 30); ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 63) == 0 && global_ns() - t0 > limit_ns) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes,
-                                              uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void grid_launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 
 // The scored columns of target rows visited mostly in increasing order: the
 // request of the last row looked up is kept, so that the next row of the same
@@ -219,23 +166,6 @@ __device__ __forceinline__ uint32_t mask_penalized(char* stage, const Desc& d, c
   drop = __reduce_or_sync(0xffffffffu, drop);
   __syncwarp();
   return drop;
-}
-
-template <int DT>
-__device__ __forceinline__ float lane_elem(const uint4& v, int q) {
-  if constexpr (DT == TT_F32) {
-    return __uint_as_float(q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w);
-  } else {
-    const int h = q >> 1;
-    const uint32_t w = h == 0 ? v.x : h == 1 ? v.y : h == 2 ? v.z : v.w;
-    return __uint_as_float((q & 1) ? (w & 0xffff0000u) : (w << 16));
-  }
-}
-
-__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
 }
 
 // Largest raw logit of one lane's share of a whole chunk. The scale is
@@ -355,18 +285,6 @@ __device__ __forceinline__ void reduce_chunk(const char* stage, const Desc& d, c
 // Candidate order of the top-k: larger logit first, then smaller column.
 __device__ __forceinline__ bool cand_before(float v1, int c1, float v2, int c2) {
   return v1 > v2 || (v1 == v2 && c1 < c2);
-}
-
-// Largest logit of one 16-byte vector (4 fp32 or 8 bf16 logits).
-template <int DT>
-__device__ __forceinline__ float vec_max(const uint4& w) {
-  if constexpr (DT == TT_F32) {
-    return fmaxf(fmaxf(__uint_as_float(w.x), __uint_as_float(w.y)),
-                 fmaxf(__uint_as_float(w.z), __uint_as_float(w.w)));
-  } else {
-    const uint32_t m = max_bf16x2(max_bf16x2(w.x, w.y), max_bf16x2(w.z, w.w));
-    return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
-  }
 }
 
 // Partial of one chunk of a nucleus row (all its columns, the scored one
@@ -1017,16 +935,20 @@ StallHook& stall_hook() {
 
 }  // namespace
 
+bool next_launch_stall(int32_t* stall_stage, uint64_t* wait_ns) {
+  StallHook& hook = stall_hook();
+  *stall_stage = -1;
+  *wait_ns = kWaitLimitNs;
+  if (hook.stall_stage < 0 || hook.launches_left.fetch_sub(1) <= 0) return false;
+  *stall_stage = hook.stall_stage;
+  *wait_ns = hook.wait_ns;
+  return true;
+}
+
 cudaError_t launch_rowpass(const RowPassArgs& args, int dt_d, int dt_t, cudaStream_t stream,
                            int sm_count, bool pdl) {
   RowPassArgs a = args;
-  a.stall_stage = -1;
-  a.wait_ns = kWaitLimitNs;
-  StallHook& hook = stall_hook();
-  if (hook.stall_stage >= 0 && hook.launches_left.fetch_sub(1) > 0) {
-    a.stall_stage = hook.stall_stage;
-    a.wait_ns = hook.wait_ns;
-  }
+  next_launch_stall(&a.stall_stage, &a.wait_ns);
   if (dt_d == TT_F32 && dt_t == TT_F32) return launch_pair<TT_F32, TT_F32>(a, stream, sm_count, pdl);
   if (dt_d == TT_F32 && dt_t == TT_BF16) return launch_pair<TT_F32, TT_BF16>(a, stream, sm_count, pdl);
   if (dt_d == TT_BF16 && dt_t == TT_F32) return launch_pair<TT_BF16, TT_F32>(a, stream, sm_count, pdl);

@@ -73,6 +73,8 @@ struct PenSizes {
 // 256-byte line, so that no single L2 address serialises every CTA's draws.
 constexpr int kWorkShards = 8;
 constexpr int kWorkStride = 32;  // in 8-byte words
+constexpr int kNucWork = 8;      // word of the first counter's line that counts the nucleus row
+                                 // kernel's rows (zeroed with the others)
 
 struct Workspace {
   Partial* part_d;   // [n_draft * nch_d]

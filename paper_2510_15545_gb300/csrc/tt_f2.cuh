@@ -53,6 +53,26 @@ __device__ __forceinline__ float exp2_scaled(float z, float scale, float M) {
   return ex2_approx(f) * __int_as_float((int(n) + 127) << 23);
 }
 
+// The normaliser of a nucleus row from its kept mass `tot` (40-bit fixed point,
+// relative to 2^M): 2^40 / tot and the natural log of tot 2^(M - 40), from fp32
+// pairs (about an ulp; fp64 is slow here). Every kernel that settles nucleus
+// rows forms them this way, so that a row's result does not depend on which did.
+constexpr float kFixScale = 1099511627776.f;  // 2^40
+struct KeptNorm {
+  float inv_tot, inv_s, lse;  // 1 / tot, 2^40 / tot
+};
+__device__ __forceinline__ KeptNorm kept_norm(unsigned long long tot, float M) {
+  const float sh = __ull2float_rn(tot);
+  const float sl = __ll2float_rn((long long)(tot - __float2ull_rn(sh)));
+  const float r = __frcp_rn(sh);
+  const float inv = fmaf(r, fmaf(-sl, r, fmaf(-sh, r, 1.f)), r);
+  const F2 l2 = two_sum(M, log2f(sh * (1.f / kFixScale)));
+  const float ln2 = 0.693147180559945f, ln2l = 1.904654299957768e-9f;
+  const float ph = __fmul_rn(l2.hi, ln2);
+  const float pl = fmaf(l2.hi, ln2, -ph) + fmaf(l2.hi, ln2l, l2.lo * ln2);
+  return {inv, inv * kFixScale, ph + pl};
+}
+
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -38,6 +38,17 @@ struct AlignArgs {
   int pairs_per_block; // (set by launch_align)
 };
 
+constexpr int kNucNarrowRows = 1;  // RowSet::nucleus
+constexpr int kNucWideRows = 2;
+// How a nucleus family's rows of V columns are settled: rows of more than
+// kNucNarrow columns (and at most kNucWideMax) by the nucleus row kernel.
+constexpr int kNucNarrow = 8192;
+constexpr int kNucWideMax = 480 * 2048;
+inline int nucleus_rows(bool nucleus, int V) {
+  if (!nucleus) return 0;
+  return V > kNucNarrow && V <= kNucWideMax ? kNucWideRows : kNucNarrowRows;
+}
+
 // One family of logits rows seen by the row pass.
 struct RowSet {
   const char* data;
@@ -51,9 +62,10 @@ struct RowSet {
   int top_k;            // > 0: filtered rows, the row pass writes top-k lists to cand
   Cand* cand;           // [n_rows * nlist * cand_stride(top_k)]: one list per row unit
   int nlist;            // units (8 KB stages: 2048 fp32 or 4096 bf16 columns) per row
-  int nucleus;          // 1: top-p without top-k (top_k = 0): the row pass writes the
-                        // compensated partials of all its columns; the nucleus
-                        // kernel finds each row's kept set
+  int nucleus;          // top-p without top-k (top_k = 0). kNucNarrowRows: the row pass
+                        // writes the compensated partials of all its columns and the
+                        // nucleus kernels find each row's kept set; kNucWideRows: the
+                        // nucleus row kernel streams the rows and finds it at once
   // Repetition penalty (top-k families only; pen = NULL: none): the row pass
   // leaves each request's penalized columns out of its unit lists, and the
   // kept-set kernel adds them back with the row's own (penalized or raw) value.
@@ -145,6 +157,24 @@ struct KeptArgs {
   int n_draft;
 };
 
+// The nucleus row kernel (nucrow.cu): the rows of families with nucleus =
+// kNucWideRows, each streamed once and its kept set found.
+struct NucRowArgs {
+  RowSet d, t;
+  int64_t rows_d, rows_t;  // rows of each such family (0: none)
+  float top_p_d, top_p_t;
+  KeptHead* head_d;
+  KeptHead* head_t;
+  float* um_d;
+  float* um_t;
+  int32_t* err;
+  int32_t epoch;
+  unsigned long long* work;  // row counter, zeroed by a grid this one depends on, or NULL:
+                             // every row belongs to a fixed share
+  int32_t stall_stage;       // as in RowPassArgs
+  uint64_t wait_ns;
+};
+
 // The repetition penalty's per-request sets (pen.cu): for each penalized
 // family, every request's history and sequence columns sorted and made unique
 // (with the first sequence position of each), and the start of each row unit.
@@ -198,6 +228,8 @@ cudaError_t launch_kept(const KeptArgs& args, cudaStream_t stream, int sm_count,
 // nucleus row from its logits and the row pass's partials, and the decision
 // over nucleus target rows.
 cudaError_t launch_nucleus(const KeptArgs& args, cudaStream_t stream, int sm_count, bool pdl);
+cudaError_t launch_nucleus_rows(const NucRowArgs& args, int dt_d, int dt_t, cudaStream_t stream,
+                                int sm_count, bool pdl);
 cudaError_t launch_decide_nucleus(const DecideArgs& args, cudaStream_t stream, bool pdl);
 cudaError_t launch_pen_prep(const PenArgs& args, cudaStream_t stream);
 cudaError_t launch_filter_q(const DecideArgs& args, cudaStream_t stream, bool pdl);
@@ -210,6 +242,11 @@ cudaError_t preload_rowpass();
 cudaError_t preload_decide();
 cudaError_t preload_filter();
 cudaError_t preload_nucleus();
+cudaError_t preload_nucleus_rows();
+
+// Test hook of the bounded waits (rowpass.cu): the stage to hold and the wait
+// limit of the next streaming launch; false (and the defaults) when off.
+bool next_launch_stall(int32_t* stall_stage, uint64_t* wait_ns);
 cudaError_t preload_pen();
 
 // Records a failed CUDA call for tt_last_cuda_error() and returns TT_ERR_CUDA.
