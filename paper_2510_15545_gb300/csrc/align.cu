@@ -22,6 +22,7 @@
 
 #include "tt_device.cuh"
 #include "tt_launch.h"
+#include "tt_f2.cuh"
 
 namespace tt {
 
@@ -751,6 +752,7 @@ __global__ void __launch_bounds__(align_threads(WPP), 1024 / align_threads(WPP))
   extern __shared__ __align__(16) char smem_raw[];
   // the row pass may start streaming target rows now; it waits for this grid
   // before it reads the needed-draft-row flags
+  if (a.after_grid) grid_dependency_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (a.work && blockIdx.x == 0 && threadIdx.x < kWorkShards)
     a.work[threadIdx.x * kWorkStride] = a.work[threadIdx.x * kWorkStride + kNucWork] =
@@ -809,6 +811,21 @@ cudaError_t preload_align() {
   return cudaSuccess;
 }
 
+template <int WPP>
+static cudaError_t launch_align_t(const AlignArgs& a, int blocks, int warps, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(unsigned(warps * 32));
+  cfg.dynamicSmemBytes = a.smem_per_pair * size_t(a.pairs_per_block);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = a.after_grid;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, align_kernel<WPP>, a);
+}
+
 cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream) {
   static int n_sm[64] = {0};
   int dev = 0;
@@ -826,11 +843,9 @@ cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream) {
     a.pairs_per_block = 1;
     const int64_t in_step = sms * std::max<int64_t>(1, kAlignRoom / int64_t(a.smem_per_pair));
     const int blocks = int(a.work ? std::min<int64_t>(a.B, in_step) : a.B);
-    if (a.max_k > 128 || a.B <= 2 * sms)
-      align_kernel<kAlignWide><<<blocks, kAlignWide * 32, a.smem_per_pair, stream>>>(a);
-    else
-      align_kernel<kAlignMid><<<blocks, kAlignMid * 32, a.smem_per_pair, stream>>>(a);
-    return cudaGetLastError();
+    return a.max_k > 128 || a.B <= 2 * sms
+               ? launch_align_t<kAlignWide>(a, blocks, kAlignWide, stream)
+               : launch_align_t<kAlignMid>(a, blocks, kAlignMid, stream);
   }
   // Small pairs: a warp each, spread over the SMs while the batch is small.
   // Before the row pass at most one CTA of kAlignWarpsStep warps per SM, whose
@@ -843,9 +858,7 @@ cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream) {
       std::max(1, std::min(most, int((a.work ? 30 * 1024 : kAlignRoom) / a.smem_per_pair)));
   const int per_pair = (a.B + a.pairs_per_block - 1) / a.pairs_per_block;
   const int blocks = a.work ? int(std::min<int64_t>(per_pair, sms)) : per_pair;
-  align_kernel<1><<<blocks, a.pairs_per_block * 32, a.smem_per_pair * size_t(a.pairs_per_block),
-                    stream>>>(a);
-  return cudaGetLastError();
+  return launch_align_t<1>(a, blocks, a.pairs_per_block, stream);
 }
 
 }  // namespace tt

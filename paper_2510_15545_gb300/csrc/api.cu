@@ -731,12 +731,13 @@ tt_status tt_step(const tt_batch* batch, const tt_vocab* vd, const tt_vocab* vt,
 
   cudaError_t e = ensure_loaded();
   if (e != cudaSuccess) return cuda_fail(e);
-  // the penalty's per-request sets, complete before the alignment (launched
-  // without a dependent-launch attribute) and so before the row pass starts
+  // the penalty's per-request sets: the alignment's CTAs wait for them, so they
+  // are complete before the row pass starts
   if ((pd || pt) &&
       (e = launch_pen_sets(batch, r.d, r.t, pd, pt, dcols, tcols, ws, s)) != cudaSuccess)
     return cuda_fail(e);
   record(prm, 0, s);
+  a.after_grid = (pd || pt) && prm->events == nullptr ? 1 : 0;
   if ((e = launch_align(a, s)) != cudaSuccess) return cuda_fail(e);
   record(prm, 1, s);
 

@@ -404,13 +404,13 @@ __device__ __forceinline__ void row_topk(const Cand* lists, int nch, int K, int 
   else row_topk_wide(lists, nch, K, Ls, lane, scr, top);
 }
 
-// The top-K of a row under the repetition penalty: its lists' top-K (which
+// The top-K of a bf16 row under the repetition penalty: its lists' top-K (which
 // leave out the request's penalized columns; -inf entries stand in for them)
 // merged with those columns, each at the row's own value: penalized (z * theta
 // for z < 0, else z / theta, fp32) when the column's first sequence position
 // lies before the row's, raw otherwise. In place in `top`; one warp.
-__device__ void penalize_top(const KeptArgs& a, const RowSet& S, int dt, bool tgt, int64_t row,
-                             int K, int lane, Cand* scr, Cand* top) {
+__device__ void penalize_top(const KeptArgs& a, const RowSet& S, bool tgt, int64_t row, int K,
+                             int lane, Cand* scr, Cand* top) {
   const int32_t* off = tgt ? a.target_off : a.draft_off;
   int lo = 0, hi = a.B - 1;
   while (lo < hi) {  // the row's request: largest b whose first row is at or before row
@@ -430,25 +430,33 @@ __device__ void penalize_top(const KeptArgs& a, const RowSet& S, int dt, bool tg
   const float tv = __shfl_sync(0xffffffffu, me.v, K - 1);
   const int tc = __shfl_sync(0xffffffffu, me.c, K - 1);
   auto value = [&](const PenEntry& e) -> float {
-    const float z = load_logit_dt(zrow, dt, e.col);
+    const float z = load_logit_dt(zrow, TT_BF16, e.col);
     return e.first < j ? (z < 0.f ? __fmul_rn(z, th) : __fdiv_rn(z, th)) : z;
   };
   __syncwarp();
   if (real) scr[lane] = me;
   int n = nt;
-  for (int i0 = 0; i0 < cnt; i0 += 32) {
-    const int i = i0 + lane;
-    Cand c = {-INFINITY, -1};
-    bool q = false;
-    if (i < cnt) {
-      const PenEntry e = S.pen[base + i];
-      c = Cand{value(e), e.col};
-      q = c.v > -INFINITY && (!full || cand_before(c.v, c.c, tv, tc));
+  // (eight entries per lane in flight: each costs two dependent accesses, the
+  // second a logit anywhere in the row)
+  constexpr int kFly = 8;
+  for (int i0 = 0; i0 < cnt; i0 += 32 * kFly) {
+    PenEntry e[kFly];
+    float z[kFly];
+#pragma unroll
+    for (int x = 0; x < kFly; ++x) {
+      const int i = i0 + 32 * x + lane;
+      e[x] = i < cnt ? S.pen[base + i] : PenEntry{-1, 0};
     }
-    const unsigned m = __ballot_sync(0xffffffffu, q);
-    const int pos = n + __popc(m & ((1u << lane) - 1u));
-    if (q && pos < kRowCap) scr[pos] = c;
-    n += __popc(m);
+#pragma unroll
+    for (int x = 0; x < kFly; ++x) z[x] = e[x].col >= 0 ? value(e[x]) : -INFINITY;
+#pragma unroll
+    for (int x = 0; x < kFly; ++x) {
+      const bool q = z[x] > -INFINITY && (!full || cand_before(z[x], e[x].col, tv, tc));
+      const unsigned m = __ballot_sync(0xffffffffu, q);
+      const int pos = n + __popc(m & ((1u << lane) - 1u));
+      if (q && pos < kRowCap) scr[pos] = Cand{z[x], e[x].col};
+      n += __popc(m);
+    }
   }
   __syncwarp();
   if (n <= kRowCap) {
@@ -539,6 +547,9 @@ __device__ __forceinline__ float kept_prob(int col, float prob, int c) {
 // draft rows skipped): the row's top-K from its unit lists, then its kept set
 // as K (probability, column) entries in value order, unused ones (0, -1),
 // and the header (lse, kept count).
+// PEN: some bf16 family has a repetition penalty (fp32 lists hold penalized
+// values already).
+template <bool PEN>
 __global__ void __launch_bounds__(kFThreads, 4) kept_kernel(KeptArgs a) {
   __shared__ Cand s_scr[kFWarps][kRowCap];
   __shared__ Cand s_top[kFWarps][TT_MAX_TOP_K];
@@ -559,8 +570,8 @@ __global__ void __launch_bounds__(kFThreads, 4) kept_kernel(KeptArgs a) {
     const int K = S.top_k;
     const int Ls = cand_stride(K);
     row_topk(S.cand + row * S.nlist * Ls, S.nlist, K, Ls, lane, s_scr[warp], s_top[warp]);
-    if (S.pen) penalize_top(a, S, tgt ? a.dt_t : a.dt_d, tgt, row, K, lane, s_scr[warp],
-                            s_top[warp]);
+    if (PEN && S.pen && (tgt ? a.dt_t : a.dt_d) == TT_BF16)
+      penalize_top(a, S, tgt, row, K, lane, s_scr[warp], s_top[warp]);
     int col;
     float prob, lse;
     const int n = kept_set(s_top[warp], K, S.scale, tgt ? a.top_p_t : a.top_p_d, lane, col,
@@ -840,7 +851,8 @@ cudaError_t launch_f(Kern kernel, int nt, const DecideArgs& args, cudaStream_t s
 cudaError_t preload_filter() {
   cudaFuncAttributes fa;
   cudaError_t e;
-  if ((e = cudaFuncGetAttributes(&fa, kept_kernel)) != cudaSuccess) return e;
+  if ((e = cudaFuncGetAttributes(&fa, kept_kernel<false>)) != cudaSuccess) return e;
+  if ((e = cudaFuncGetAttributes(&fa, kept_kernel<true>)) != cudaSuccess) return e;
   if ((e = cudaFuncGetAttributes(&fa, filter_q_kernel<128>)) != cudaSuccess) return e;
   if ((e = cudaFuncGetAttributes(&fa, filter_q_kernel<256>)) != cudaSuccess) return e;
   if ((e = cudaFuncGetAttributes(&fa, decide_filtered_kernel<128>)) != cudaSuccess) return e;
@@ -862,7 +874,9 @@ cudaError_t launch_kept(const KeptArgs& args, cudaStream_t stream, int sm_count,
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kept_kernel, args);
+  const bool pen = (args.d.pen && args.dt_d == TT_BF16) || (args.t.pen && args.dt_t == TT_BF16);
+  return pen ? cudaLaunchKernelEx(&cfg, kept_kernel<true>, args)
+             : cudaLaunchKernelEx(&cfg, kept_kernel<false>, args);
 }
 
 // 128 threads per request when the batch has more than four requests per SM

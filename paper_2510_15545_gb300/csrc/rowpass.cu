@@ -141,31 +141,71 @@ __device__ __forceinline__ int req_lookup(const int32_t* off, int B, bool tgt, R
   return (r >= r0 && r <= r1) ? b : -1;
 }
 
-// Repetition penalty: the request's penalized columns within a unit held in
-// shared memory are set to -inf (they leave its top-k list; the kept-set
-// kernel adds them back with the row's own values); those in the unit's
-// ragged tail, read directly, are returned as lane bits to drop.
-template <int DT>
-__device__ __forceinline__ uint32_t mask_penalized(char* stage, const Desc& d, const RowSet& S,
-                                                   int cps, int lane) {
-  const int u = d.chunk / cps;
-  const int64_t srow = int64_t(d.req) * (S.nch + 1);
+// Repetition penalty: where a unit's penalized columns lie, and the first 32
+// of them, one per lane. A consumer warp loads them for the unit that it will
+// most likely take next, kConsumerWarps further on in the row, while it works
+// on the current one: each is two dependent accesses, of a microsecond and more
+// beside the streaming row pass, which a warp would wait for on every unit.
+struct PenUnit {
+  int64_t row;      // 2 * row + family; -1: none
+  int32_t unit;
+  int32_t lo, hi;   // the unit's entries
+  int32_t pos;      // the row's position in its request
+  PenEntry e;       // this lane's entry (lo + lane); column -1: none
+};
+
+// First half: the unit's range of entries.
+__device__ __forceinline__ PenUnit pen_range(const RowPassArgs& a, const Desc& d, int unit) {
+  const RowSet& S = d.set ? a.t : a.d;
+  const int64_t at = int64_t(d.req) * (S.nch + 1) + unit;
   const int base = S.pbase[d.req];
-  const int lo = S.pstart[srow + u], hi = S.pstart[srow + u + 1];
+  const int64_t first = d.set ? int64_t(a.target_off[d.req]) + d.req : a.draft_off[d.req];
+  return {d.row * 2 + d.set, unit, base + S.pstart[at], base + S.pstart[at + 1],
+          int32_t(d.row - first), {-1, 0}};
+}
+// Second half: its first entries.
+__device__ __forceinline__ void pen_entries(PenUnit& p, const RowSet& S, int lane) {
+  if (p.row >= 0 && p.lo + lane < p.hi) p.e = S.pen[p.lo + lane];
+}
+
+// Logit z penalized by theta (first position `first` of its column, row `pos`).
+__device__ __forceinline__ float penalized(float z, float theta, bool on) {
+  return on ? (z < 0.f ? __fmul_rn(z, theta) : __fdiv_rn(z, theta)) : z;
+}
+
+// The request's penalized columns within a unit held in shared memory. An fp32
+// unit takes the row's own values in place (NaN: -inf), so that its list is
+// final. A bf16 unit cannot hold them: the columns are set to -inf (they leave
+// the list) and the kept-set kernel adds them back. Columns of the unit's
+// ragged tail, read directly, are returned as lane bits: bf16 ones to drop;
+// fp32 ones as penalized (bit 0 + lane) or listed (bit 16 + lane).
+// (64 requests, fp32 rows of 152 k columns, histories of 64 to 1024: with both
+// families added back by the kept-set kernel, which reads every penalized logit
+// of a row again, 8 loads in flight per lane, a step took 204 us; in place 143.)
+template <int DT>
+__device__ __forceinline__ uint32_t apply_penalty(char* stage, const Desc& d, const RowSet& S,
+                                                  const PenUnit& p, int lane) {
   const int c0 = d.chunk * kChunk;
-  uint32_t drop = 0u;
-  for (int i = lo + lane; i < hi; i += 32) {
-    const int x = S.pen[base + i].col - c0;
+  uint32_t tail = 0u;
+  auto apply = [&](const PenEntry& e) {
+    const int x = e.col - c0;
     if (x >= 0 && x < d.n_smem) {
-      if constexpr (DT == TT_F32) reinterpret_cast<float*>(stage)[x] = -INFINITY;
-      else reinterpret_cast<uint16_t*>(stage)[x] = 0xff80u;  // bf16 -inf
+      if constexpr (DT == TT_F32) {
+        float* z = reinterpret_cast<float*>(stage) + x;
+        *z = fmaxf(penalized(*z, S.penalty, e.first < p.pos), -INFINITY);  // (NaN: -inf)
+      } else {
+        reinterpret_cast<uint16_t*>(stage)[x] = 0xff80u;  // bf16 -inf
+      }
     } else if (x >= d.n_smem && x < d.n) {
-      drop |= 1u << (x - d.n_smem);
+      const int l = x - d.n_smem;
+      tail |= DT == TT_F32 ? (0x10000u << l) | (e.first < p.pos ? 1u << l : 0u) : 1u << l;
     }
-  }
-  drop = __reduce_or_sync(0xffffffffu, drop);
+  };
+  if (p.e.col >= 0) apply(p.e);
+  for (int i = p.lo + 32 + lane; i < p.hi; i += 32) apply(S.pen[i]);
+  tail = __reduce_or_sync(0xffffffffu, tail);
   __syncwarp();
-  return drop;
+  return tail;
 }
 
 // Largest raw logit of one lane's share of a whole chunk. The scale is
@@ -356,7 +396,7 @@ __device__ __forceinline__ Partial nuc_chunk_partial(const char* stage, const De
 // every unit, which keeps the stage ring from waiting on one slow warp.
 template <int DT>
 __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, int lane, int K,
-                            Cand* scratch, Cand* out, uint32_t tail_drop = 0u) {
+                            Cand* scratch, Cand* out, uint32_t tail_pen = 0u) {
   constexpr int VEC = DT == TT_F32 ? 4 : 8;  // logits per 16-byte vector
   constexpr int NV = kChunk * 4 / (16 * 32);   // vectors per lane in one stage
   constexpr uint32_t kTailBit = 1u << NV;      // flag of the lane's tail element
@@ -366,11 +406,15 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
   const int nvec = d.n_smem / VEC;  // whole vectors delivered (the copy moves 16-byte units)
   // this lane's vectors v < nvl lie within the copy
   const int nvl = max(0, min(NV, (nvec - lane + 31) >> 5));
-  const bool has_tail = lane < d.n - d.n_smem && !((tail_drop >> lane) & 1u);
+  bool has_tail = lane < d.n - d.n_smem && !(DT == TT_BF16 && ((tail_pen >> lane) & 1u));
   // the tail element, NaN where the lane has none (NaN never compares >=)
   float zt = kNaN;
   if (has_tail) {
     zt = load_logit<DT>(S.row(d), int64_t(col0) + d.n_smem + lane);
+    if (DT == TT_F32 && ((tail_pen >> lane) & 0x10000u)) {
+      zt = penalized(zt, (d.set ? S.a.t : S.a.d).penalty, (tail_pen >> lane) & 1u);
+      has_tail = zt == zt;
+    }
   }
   const uint32_t valid = ((1u << nvl) - 1) | (has_tail ? kTailBit : 0u);
   float vm[NV];  // vector maxima; -inf for a vector past the copy
@@ -729,6 +773,7 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
   // (one thread's launch_dependents counts for its whole CTA: only the
   // producer lane gives it, after its grid-dependency wait, because the next
   // grid reads the alignment's outputs before its own wait)
+  PenUnit pu = {-1, 0, 0, 0, 0, {-1, 0}};  // the unit expected next (penalized rows)
   for (int it = warp;; it += kConsumerWarps) {
     const int s = it % R::kStages;
     const uint32_t par = (it / R::kStages) & 1;
@@ -763,21 +808,29 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
       const RowSet& S = d.set ? a.t : a.d;
       Cand* out = S.cand + (d.row * S.nlist + d.chunk / cps) * cand_stride(S.top_k);
       const RowView V = {a, S.scale};
-      uint32_t drop = 0u;
+      uint32_t tail_pen = 0u;
       if constexpr (SEL == 2) {
         if (S.pen && d.req >= 0) {
           char* wstage = stages + size_t(s) * R::kStageBytes;
-          drop = (d.set ? DTT : DTD) == TT_F32 ? mask_penalized<TT_F32>(wstage, d, S, cps, lane)
-                                               : mask_penalized<TT_BF16>(wstage, d, S, cps, lane);
+          const int unit = d.chunk / cps;
+          if (pu.row != d.row * 2 + d.set || pu.unit != unit) {
+            pu = pen_range(a, d, unit);
+            pen_entries(pu, S, lane);
+          }
+          tail_pen = (d.set ? DTT : DTD) == TT_F32 ? apply_penalty<TT_F32>(wstage, d, S, pu, lane)
+                                                   : apply_penalty<TT_BF16>(wstage, d, S, pu, lane);
+          pu.row = -1;
+          if (unit + kConsumerWarps < S.nlist) pu = pen_range(a, d, unit + kConsumerWarps);
         }
       }
       if constexpr (DTD == DTT) {
-        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, drop);
+        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
       } else if (d.set) {
-        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, drop);
+        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
       } else {
-        select_unit<DTD>(stage, d, V, lane, S.top_k, scratch, out, drop);
+        select_unit<DTD>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
       }
+      if (SEL == 2 && S.pen && d.req >= 0) pen_entries(pu, S, lane);
       if (lane == 0 && !(blockIdx.x == 0 && it == a.stall_stage))
         mbar_arrive(&empty[s]);  // the stage's bytes are consumed
       continue;
@@ -883,7 +936,7 @@ cudaError_t preload_pair() {
 }
 
 // Variants: 0 partials only; 1 top-k lists for filtered families; 2 lists with
-// the repetition penalty's masking and the nucleus rows' partials (kept apart
+// the repetition penalty and the nucleus rows' partials (kept apart
 // so that plain filtered rows run the smaller consumer loop).
 template <int DTD, int DTT>
 cudaError_t launch_pair(const RowPassArgs& a, cudaStream_t stream, int sm_count, bool pdl) {

@@ -57,7 +57,7 @@ struct KeptHead {
 // A column of a request's repetition-penalty set (its history and sequence
 // tokens): the column and the first sequence position holding it (-1 when the
 // history holds it), so that a row at position j penalizes it when first < j.
-// A request's entries are sorted by column, one per column.
+// A request's entries are grouped by row unit, one per column.
 struct PenEntry {
   int32_t col;
   int32_t first;
@@ -95,9 +95,9 @@ struct Workspace {
   KeptHead* head_t;  // [n_target + B]
   float* um_d;       // [n_draft * nch_d] kept probability mass per chunk of nucleus draft rows
   float* um_t;       // [(n_target + B) * nch_t] the same for nucleus target rows
-  // repetition penalty, per penalized family: each request's sorted penalized
-  // columns (at base[b], cnt[b] entries, capacity its history plus its tokens)
-  // and, per row unit u, the first entry at or past the unit's first column
+  // repetition penalty, per penalized family: each request's penalized columns
+  // by row unit (at base[b], cnt[b] entries, capacity its history plus its tokens)
+  // and, per row unit u, its first entry
   PenEntry* pen_d;    // [n_hist_d + n_draft]
   int32_t* pbase_d;   // [B]
   int32_t* pcnt_d;    // [B]

@@ -33,6 +33,8 @@ struct AlignArgs {
   const int32_t* target_cols;  // scored column of each target position
   int32_t* excl;               // [n_target + B] written: scored column of each target row
                                // (-1 for the bonus row), may be NULL
+  int after_grid;      // 1: launched while the grid before it (the penalty's sets) may run;
+                       // the row pass, which reads those, starts after both
   int tile_blocks;     // 16-byte blocks of a pair's cost tile
   size_t smem_per_pair;
   int pairs_per_block; // (set by launch_align)
@@ -67,9 +69,10 @@ struct RowSet {
                         // nucleus kernels find each row's kept set; kNucWideRows: the
                         // nucleus row kernel streams the rows and finds it at once
   // Repetition penalty (top-k families only; pen = NULL: none): the row pass
-  // leaves each request's penalized columns out of its unit lists, and the
-  // kept-set kernel adds them back with the row's own (penalized or raw) value.
-  const PenEntry* pen;    // sorted penalized columns of request b at pbase[b] (pcnt[b])
+  // gives each request's penalized columns the row's own (penalized or raw)
+  // value in fp32 units; bf16 units leave them out of their lists and the
+  // kept-set kernel adds them back.
+  const PenEntry* pen;    // penalized columns of request b at pbase[b] (pcnt[b]), by unit
   const int32_t* pbase;
   const int32_t* pcnt;
   const int32_t* pstart;  // [B * (nch + 1)]: first entry of each row unit, then pcnt
@@ -176,8 +179,8 @@ struct NucRowArgs {
 };
 
 // The repetition penalty's per-request sets (pen.cu): for each penalized
-// family, every request's history and sequence columns sorted and made unique
-// (with the first sequence position of each), and the start of each row unit.
+// family, every request's history and sequence columns, one entry each (with
+// its first sequence position), by row unit, and the start of each unit.
 struct PenArgs {
   int B;
   int on_d, on_t;

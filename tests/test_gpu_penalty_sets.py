@@ -1,0 +1,80 @@
+"""The repetition penalty's per-request sets (one entry per column, grouped by
+row unit) and the two ways a row takes them (fp32 units in place, bf16 units
+left out and added back), at the sizes where they can go wrong, against the
+oracle: counts around a warp and at the cap, one column repeated, a whole unit
+penalized, ragged tails, families of different types."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_15545_gb300 as tt
+from paper_2510_15545_gb300 import workload as W
+from _parity import compare, oracle_step, to_np
+
+pytestmark = pytest.mark.gpu
+PEN = dict(temp_draft=0.7, temp_target=0.7, top_k_draft=20, top_p_draft=0.8, top_k_target=20,
+           top_p_target=0.8, rep_penalty_draft=1.1, rep_penalty_target=1.3)
+CAP = 3072  # columns of a history
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    tt.load(build_if_missing=True)
+
+
+def _padded(t):
+    """Rows padded to 16 bytes plus one more vector, the padding NaN."""
+    R, V = t.shape
+    per16 = 16 // t.element_size()
+    buf = torch.full((R, (V + per16 - 1) // per16 * per16 + per16), float("nan"),
+                     dtype=t.dtype, device="cuda")
+    buf[:, :V] = t.to("cuda")
+    return buf[:, :V]
+
+
+def _histories(V, top, rng):
+    """One history per request: the shapes named above, each with the rows' own
+    leading columns (which decide the lists)."""
+    tail = np.arange(V - 9, V)
+    unit = np.arange(2048, min(4096 + 5, V)) if V > 2048 else np.arange(V)
+    shapes = [np.array([], np.int64), rng.integers(0, V, 1), rng.integers(0, min(V, 2048), 31),
+              rng.integers(0, min(V, 2048), 32), rng.integers(0, min(V, 2048), 33),
+              np.full(CAP, V - 1), rng.integers(0, V, CAP), np.concatenate([tail, tail[::-1]]),
+              unit, rng.permutation(V)[:CAP]]
+    return [np.concatenate([s, top[i]])[-CAP:] if i else s for i, s in enumerate(shapes)]
+
+
+@pytest.mark.parametrize("V", [257, 4099, 20011])
+@pytest.mark.parametrize("dt_d,dt_t", [(torch.float32, torch.float32),
+                                       (torch.bfloat16, torch.bfloat16),
+                                       (torch.float32, torch.bfloat16),
+                                       (torch.bfloat16, torch.float32)])
+@pytest.mark.parametrize("families", ["both", "draft", "target"])
+def test_sets_at_edges(V, dt_d, dt_t, families):
+    B, G = 10, 4
+    wl = W.homogeneous_workload(B, G, V, seed=V, logit_scale=2.5)
+    wl = dataclasses.replace(wl, draft_logits=wl.draft_logits.to(dt_d),
+                             target_logits=wl.target_logits.to(dt_t))
+    rng = np.random.default_rng(V)
+    h = {}
+    for fam, logits in (("d", wl.draft_logits), ("t", wl.target_logits)):
+        lead = torch.topk(logits.float().reshape(B, -1, V), 6, dim=2).indices.reshape(B, -1)
+        hs = _histories(logits.shape[1], lead.numpy(), rng)
+        h["hist_off_" + fam] = np.concatenate([[0], np.cumsum([len(x) for x in hs])]).astype(np.int32)
+        h["hist_cols_" + fam] = np.concatenate(hs).astype(np.int32)
+    wl = dataclasses.replace(wl, **h)
+    f = dict(PEN)
+    if families == "draft":
+        f["rep_penalty_target"] = 1.0
+    if families == "target":
+        f["rep_penalty_draft"] = 1.0
+    inp = tt.device_inputs(wl, "cuda")
+    for k, v in f.items():
+        setattr(inp["params"], k, v)
+    g = to_np(tt.tt_step(inp["batch"], inp["vd"], inp["vt"], _padded(wl.draft_logits),
+                         _padded(wl.target_logits), inp["params"]))
+    compare(wl, g, oracle_step(wl, **f))
