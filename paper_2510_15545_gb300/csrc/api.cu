@@ -903,19 +903,18 @@ tt_status tt_verify_sharded(const tt_batch* batch, const float* q_hat, const tt_
     d.part = ws.part[k];
   }
   if ((e = launch_shard_excl(a, s)) != cudaSuccess) return cuda_fail(e);
-  // each shard's slice reduced by its own row pass (what one rank does). Passes
-  // after the first start while the one before drains (programmatic dependent
-  // launch): what they read before their grid-dependency wait -- the scored
-  // columns and their zeroed work counters -- was written by the excl kernel,
-  // which finished before the first pass, launched without the attribute, began.
-  for (int k = 0; k < target->S; ++k) {
-    RowPassArgs r;
+  // The shards' slices (what the ranks do), those of one type in one row pass.
+  // Each kernel from here on starts while the one before drains (programmatic
+  // dependent launch) and waits for it before it reads what it wrote.
+  int pass = 0;
+  for (int dt : {TT_F32, TT_BF16}) {
+    ShardPassArgs r;
     std::memset(&r, 0, sizeof r);
-    r.t = rowset(&target->shards[k], ws.part[k], nullptr, prm->temp_target);
-    r.rows_t = rows;
     r.d = no_rows();
-    r.rows_d = 0;
-    r.excl = ws.excl + int64_t(k) * rows;
+    r.t = no_rows();
+    r.t.V = V;
+    r.t.scale = a.scale;
+    r.rows_t = rows;
     r.B = batch->B;
     r.n_target = batch->n_target;
     r.target_off = batch->target_off;
@@ -923,11 +922,16 @@ tt_status tt_verify_sharded(const tt_batch* batch, const float* q_hat, const tt_
     r.err = ws.err;
     r.epoch = a.epoch;
     r.pre_eighths = 4;
+    for (int k = 0; k < target->S; ++k) {
+      if (a.sh[k].dtype != dt) continue;
+      const ShardDesc& d = a.sh[k];
+      r.sh[r.S++] = {d.data, d.stride_bytes, target->shards[k].n_rows, d.part,
+                     ws.excl + int64_t(k) * rows, 0, d.V, d.col0, d.nch};
+    }
+    if (r.S == 0) continue;
     r.work = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ws.work) +
-                                                   size_t(k) * kWorkShards * kWorkStride *
-                                                       sizeof(unsigned long long));
-    if ((e = launch_rowpass(r, target->shards[k].dtype, target->shards[k].dtype, s,
-                            sm_count_current(), k > 0)) != cudaSuccess)
+                                                   kShardWorkBytes * pass++);
+    if ((e = launch_shard_rowpass(r, dt, s, sm_count_current(), true)) != cudaSuccess)
       return cuda_fail(e);
   }
   if ((e = launch_shard_summary(a, s, sm_count_current())) != cudaSuccess) return cuda_fail(e);
@@ -935,7 +939,7 @@ tt_status tt_verify_sharded(const tt_batch* batch, const float* q_hat, const tt_
       (e = cudaMemcpyAsync(summaries, ws.rec, sizeof(ShardRec) * size_t(target->S) * rows,
                            cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
     return cuda_fail(e);
-  if ((e = launch_decide_sharded(a, s)) != cudaSuccess) return cuda_fail(e);
+  if ((e = launch_decide_sharded(a, s, !summaries)) != cudaSuccess) return cuda_fail(e);
   return TT_OK;
 }
 

@@ -49,6 +49,11 @@ struct Desc {
 // Stage s is always refilled for the same consumer warp (s mod kConsumerWarps),
 // so a warp never waits on a stage more than one phase ahead of it: an
 // mbarrier parity wait cannot tell phase n from phase n + 2.
+// The variant that takes column shards of the target rows: all shards of one
+// type in one grid, so that one ring fill and one tail serve them all. Four
+// shards of 64 requests (415 MB) took four passes of 23 us in turn, 68 us now.
+constexpr int kShards = 3;
+
 constexpr int kCandCap = 128;   // top-k candidates of one unit a warp keeps in shared memory
 constexpr int kDirectCap = 32;  // vectors at or above tau1 taken directly (more: tau2)
 constexpr int kLevel2Cap = 64;  // vector maxima ranked by counting (more: radix search)
@@ -59,7 +64,8 @@ struct Ring {
   static constexpr int kCpsD = DTD == TT_F32 ? 1 : 2;  // chunks per stage, draft rows
   static constexpr int kCpsT = DTT == TT_F32 ? 1 : 2;  // chunks per stage, target rows
   static constexpr int kStages = kRingBytes / kStageBytes;
-  static constexpr size_t kScratch = SEL ? size_t(kConsumerWarps) * kCandCap * sizeof(Cand) : 0;
+  static constexpr bool kLists = SEL == 1 || SEL == 2;
+  static constexpr size_t kScratch = kLists ? size_t(kConsumerWarps) * kCandCap * sizeof(Cand) : 0;
   static constexpr size_t kSmem =
       size_t(kRingBytes) + kStages * (2 * sizeof(uint64_t) + sizeof(Desc)) + kScratch;
   static_assert(kStages % kConsumerWarps == 0, "each stage belongs to one consumer warp");
@@ -246,6 +252,13 @@ struct RowView {
     return d.set ? a.t.data + d.row * a.t.stride_bytes : a.d.data + d.row * a.d.stride_bytes;
   }
 };
+struct ShardView {  // d.set: 1 + the shard
+  const ShardPassArgs& a;
+  float scale;
+  __device__ __forceinline__ const char* row(const Desc& d) const {
+    return a.sh[d.set - 1].data + d.row * a.sh[d.set - 1].stride_bytes;
+  }
+};
 
 // One consumer warp reduces one chunk held in shared memory (plus a ragged
 // tail of fewer than 16 bytes read directly) to (max, sum of 2^(s - max)).
@@ -295,8 +308,8 @@ __device__ __noinline__ float2 reduce_stage_edge(const uint4* sv, int n_smem, in
   return make_float2(mx, sum);
 }
 
-template <int DT>
-__device__ __forceinline__ void reduce_chunk(const char* stage, const Desc& d, const RowView& S,
+template <int DT, typename View>
+__device__ __forceinline__ void reduce_chunk(const char* stage, const Desc& d, const View& S,
                                              int lane, float& m_out, float& s_out) {
   const uint4* sv = reinterpret_cast<const uint4*>(stage);
   const float scale = S.scale;
@@ -580,8 +593,12 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
   __syncwarp();  // the scratch is free for the next unit
 }
 
+template <int SEL>
+using PassArgs = std::conditional_t<SEL == kShards, ShardPassArgs, RowPassArgs>;
+
 template <int DTD, int DTT, int SEL>
-__global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
+__global__ void __launch_bounds__(kThreads, 3)
+    rowpass_kernel(const __grid_constant__ PassArgs<SEL> a) {
   using R = Ring<DTD, DTT, SEL>;
   extern __shared__ __align__(128) char smem[];
   char* stages = smem;
@@ -590,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
   Desc* desc = reinterpret_cast<Desc*>(empty + R::kStages);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // a consumer warp's candidate scratch (filtered rows only)
-  Cand* scratch = reinterpret_cast<Cand*>(desc + R::kStages) + (SEL ? warp * kCandCap : 0);
+  Cand* scratch = reinterpret_cast<Cand*>(desc + R::kStages) + (R::kLists ? warp * kCandCap : 0);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < R::kStages; ++s) {
@@ -608,30 +625,52 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
       // units (stages) per row and in all of each family
       const int upr_t = (a.t.nch + R::kCpsT - 1) / R::kCpsT;
       const int upr_d = (a.d.nch + R::kCpsD - 1) / R::kCpsD;
-      const int64_t items_t = a.rows_t * upr_t, items_d = a.rows_d * upr_d;
+      int64_t items_t = a.rows_t * upr_t;
+      if constexpr (SEL == kShards) items_t = a.sh[a.S - 1].end;
+      const int64_t items_d = a.rows_d * upr_d;
       bool ok = true;
       int it = 0;
       int64_t cached_row = -1, cached_drow = -1;
-      int cached_excl = -1;
+      int cached_excl = -1, cached_set = 0;
       __shared__ ExclCursor cursor;
       __shared__ ReqCursor rcur_d, rcur_t;
       cursor.b = -1;
       rcur_d.b = rcur_t.b = -1;
       bool cached_need = true;
-      // Queues chunk `chunk` of row `row` (tgt: a target row, else a draft
-      // row) on the next stage; false once a wait has run out.
+      // Queues unit `unit` of row `row` of a family (set 0: draft rows, 1: target
+      // rows; shards: 1 + the shard) on the next stage; false once a wait has run out.
       bool late = false;  // past the grid-dependency wait
-      auto issue = [&](bool tgt, int64_t row, int unit) -> bool {
+      auto issue = [&](int set, int64_t row, int unit) -> bool {
+        const bool tgt = set != 0;
         Desc d;
-        const RowSet* S;
+        const RowSet* S = tgt ? &a.t : &a.d;
+        const char* base = S->data;
+        int64_t stride = S->stride_bytes, n_rows = S->n_rows;
+        int V = S->V;
         int esz, cps;
         d.row = row;
+        d.set = set;
+        if constexpr (SEL == kShards) {
+          const ShardRows& H = a.sh[set - 1];
+          base = H.data;
+          stride = H.stride_bytes;
+          n_rows = H.n_rows;
+          V = H.V;
+          if (row != cached_row || set != cached_set) {
+            cached_row = row;
+            cached_set = set;
+            if (late) {
+              cached_excl = H.excl[row];
+            } else {
+              const int c = excl_lookup(a, &cursor, row), x = c - H.col0;
+              cached_excl = (c >= 0 && x >= 0 && x < V) ? x : -1;
+            }
+          }
+        }
         if (tgt) {
-          S = &a.t;
           esz = DTT == TT_F32 ? 4 : 2;
           cps = R::kCpsT;
-          d.set = 1;
-          if (row != cached_row) {
+          if (SEL != kShards && row != cached_row) {
             cached_row = row;
             cached_excl = a.excl                ? a.excl[row]
                           : (late && a.excl_late) ? a.excl_late[row]
@@ -640,10 +679,8 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
           const int ex = cached_excl - unit * cps * kChunk;
           d.excl = (cached_excl >= 0 && ex >= 0 && ex < cps * kChunk) ? ex : -1;
         } else {
-          S = &a.d;
           esz = DTD == TT_F32 ? 4 : 2;
           cps = R::kCpsD;
-          d.set = 0;
           d.excl = -1;
           if (row != cached_drow) {
             cached_drow = row;
@@ -657,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
                                      : -1;
         d.chunk = unit * cps;
         const int c0 = d.chunk * kChunk;
-        d.n = min(cps * kChunk, S->V - c0);
+        d.n = min(cps * kChunk, V - c0);
         const uint32_t bytes = uint32_t(d.n * esz) & ~15u;  // bulk copies move 16-byte units
         d.n_smem = int(bytes) / esz;
         const int s = it % R::kStages;
@@ -667,8 +704,8 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
           return false;
         }
         // every bulk copy is checked against the tensor before it is issued
-        const char* src = S->data + d.row * S->stride_bytes + size_t(c0) * esz;
-        const bool copy_ok = d.row >= 0 && d.row < S->n_rows && c0 >= 0 && d.n > 0 &&
+        const char* src = base + d.row * stride + size_t(c0) * esz;
+        const bool copy_ok = d.row >= 0 && d.row < n_rows && c0 >= 0 && d.n > 0 &&
                              (reinterpret_cast<uintptr_t>(src) & 15) == 0 &&
                              bytes <= uint32_t(R::kStageBytes);
         if (!copy_ok) {
@@ -690,14 +727,26 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
       // walking rows and units without a division per item.
       auto walk = [&](bool tgt, int64_t i0, int64_t i1) {
         if (i0 >= i1) return;
-        const int upr = tgt ? upr_t : upr_d;
-        int64_t row = i0 / upr;
-        int unit = int(i0 - row * upr);
+        int set = tgt ? 1 : 0;
+        int upr = tgt ? upr_t : upr_d;
+        int64_t first = 0;
+        if constexpr (SEL == kShards) {
+          while (set < a.S && i0 >= a.sh[set - 1].end) first = a.sh[set++ - 1].end;
+          upr = (a.sh[set - 1].nch + R::kCpsT - 1) / R::kCpsT;
+        }
+        int64_t row = (i0 - first) / upr;
+        int unit = int(i0 - first - row * upr);
         for (int64_t i = i0; ok && i < i1; ++i) {
-          ok = issue(tgt, row, unit);
+          ok = issue(set, row, unit);
           if (++unit == upr) {
             unit = 0;
             ++row;
+            if constexpr (SEL == kShards) {
+              if (row == a.rows_t && set < a.S) {
+                row = 0;
+                upr = (a.sh[set++].nch + R::kCpsT - 1) / R::kCpsT;
+              }
+            }
           }
         }
       };
@@ -804,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
         continue;
       }
     }
-    if (SEL && (d.set ? a.t : a.d).top_k > 0) {  // filtered rows: the unit's top-k list
+    if (R::kLists && (d.set ? a.t : a.d).top_k > 0) {  // filtered rows: the unit's top-k list
       const RowSet& S = d.set ? a.t : a.d;
       Cand* out = S.cand + (d.row * S.nlist + d.chunk / cps) * cand_stride(S.top_k);
       const RowView V = {a, S.scale};
@@ -850,7 +899,9 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
       float mc = -INFINITY, sc = 0.f;
       // fp32 rows: one copy for both families; bf16 rows: one per family (shared,
       // the kernel needs more registers than the decision kernel beside it leaves)
-      if constexpr (DTD == TT_F32 && DTT == TT_F32) {
+      if constexpr (SEL == kShards) {
+        reduce_chunk<DTT>(stage + size_t(lo) * esz, e, ShardView{a, a.t.scale}, lane, mc, sc);
+      } else if constexpr (DTD == TT_F32 && DTT == TT_F32) {
         reduce_chunk<TT_F32>(stage + size_t(lo) * esz, e,
                              RowView{a, d.set ? a.t.scale : a.d.scale}, lane, mc, sc);
       } else if (d.set) {
@@ -871,13 +922,19 @@ __global__ void __launch_bounds__(kThreads, 3) rowpass_kernel(RowPassArgs a) {
     // it, so the producer's bounded wait for it runs out, then the others')
     if (lane == 0 && !(blockIdx.x == 0 && it == a.stall_stage))
       mbar_arrive(&empty[s]);  // the stage's bytes are consumed
-    const RowSet& S = d.set ? a.t : a.d;
     if (d.n <= 0) continue;  // nothing copied (a failed check: the row may not exist)
+    Partial* part;
+    if constexpr (SEL == kShards) {
+      part = a.sh[d.set - 1].part + d.row * a.sh[d.set - 1].nch + d.chunk;
+    } else {
+      const RowSet& S = d.set ? a.t : a.d;
+      part = S.part + d.row * S.nch + d.chunk;
+    }
     warp_merge_ms(m0, s0);
-    if (lane == 0) S.part[d.row * S.nch + d.chunk] = Partial{m0, s0};
+    if (lane == 0) part[0] = Partial{m0, s0};
     if (cps > 1 && kChunk < d.n) {
       warp_merge_ms(m1, s1);
-      if (lane == 0) S.part[d.row * S.nch + d.chunk + 1] = Partial{m1, s1};
+      if (lane == 0) part[1] = Partial{m1, s1};
     }
   }
 }
@@ -907,12 +964,14 @@ cudaError_t preload_t() {
 }
 
 template <int DTD, int DTT, int SEL>
-cudaError_t launch_rowpass_t(const RowPassArgs& a, cudaStream_t stream, int sm_count, bool pdl) {
+cudaError_t launch_rowpass_t(const PassArgs<SEL>& a, cudaStream_t stream, int sm_count,
+                             bool pdl) {
   using R = Ring<DTD, DTT, SEL>;
   const int per_sm = resident_per_sm<DTD, DTT, SEL>();
   if (per_sm == 0) return cudaErrorNotReady;  // preload_rowpass() was not called
-  const int64_t total = a.rows_t * ((a.t.nch + R::kCpsT - 1) / R::kCpsT) +
-                        a.rows_d * ((a.d.nch + R::kCpsD - 1) / R::kCpsD);
+  int64_t total = a.rows_t * ((a.t.nch + R::kCpsT - 1) / R::kCpsT) +
+                  a.rows_d * ((a.d.nch + R::kCpsD - 1) / R::kCpsD);
+  if constexpr (SEL == kShards) total = a.sh[a.S - 1].end;
   if (total == 0) return cudaSuccess;
   const int64_t grid = std::min<int64_t>(total, int64_t(sm_count) * per_sm);
   cudaLaunchConfig_t cfg = {};
@@ -953,6 +1012,8 @@ cudaError_t preload_rowpass() {
   if ((e = preload_pair<TT_F32, TT_F32>()) != cudaSuccess) return e;
   if ((e = preload_pair<TT_F32, TT_BF16>()) != cudaSuccess) return e;
   if ((e = preload_pair<TT_BF16, TT_F32>()) != cudaSuccess) return e;
+  if ((e = preload_t<TT_F32, TT_F32, kShards>()) != cudaSuccess) return e;
+  if ((e = preload_t<TT_BF16, TT_BF16, kShards>()) != cudaSuccess) return e;
   return preload_pair<TT_BF16, TT_BF16>();
 }
 
@@ -1006,6 +1067,20 @@ cudaError_t launch_rowpass(const RowPassArgs& args, int dt_d, int dt_t, cudaStre
   if (dt_d == TT_F32 && dt_t == TT_BF16) return launch_pair<TT_F32, TT_BF16>(a, stream, sm_count, pdl);
   if (dt_d == TT_BF16 && dt_t == TT_F32) return launch_pair<TT_BF16, TT_F32>(a, stream, sm_count, pdl);
   return launch_pair<TT_BF16, TT_BF16>(a, stream, sm_count, pdl);
+}
+
+cudaError_t launch_shard_rowpass(const ShardPassArgs& args, int dt, cudaStream_t stream,
+                                 int sm_count, bool pdl) {
+  ShardPassArgs a = args;
+  next_launch_stall(&a.stall_stage, &a.wait_ns);
+  const int cps = dt == TT_F32 ? 1 : 2;
+  int64_t end = 0;
+  for (int k = 0; k < a.S; ++k) {
+    end += a.rows_t * ((a.sh[k].nch + cps - 1) / cps);
+    a.sh[k].end = end;
+  }
+  return dt == TT_F32 ? launch_rowpass_t<TT_F32, TT_F32, kShards>(a, stream, sm_count, pdl)
+                      : launch_rowpass_t<TT_BF16, TT_BF16, kShards>(a, stream, sm_count, pdl);
 }
 
 }  // namespace tt

@@ -2,8 +2,9 @@
 // target rows split by columns into S shards, as a tensor-parallel target
 // model leaves them, emulated on one GPU.
 //
-// Per shard (what one rank does with its slice): a row pass over the slice
-// gives chunk partials with the scored token left out; shard_summary_kernel
+// A row pass over the slices (one grid for all shards of a type; per shard it is
+// what one rank does) gives chunk partials with the scored token left out;
+// shard_summary_kernel
 // reduces them to one record per row (max, sum of 2^(s - max) as an fp64 pair
 // of floats, the owned scored token's scaled logit or NaN). The records of all
 // shards are the exchange (an all-gather across ranks; here a device buffer in
@@ -18,6 +19,7 @@
 #include <cstring>
 
 #include "tt_device.cuh"
+#include "tt_f2.cuh"
 #include "tt_launch.h"
 #include "tt_shard.h"
 
@@ -26,6 +28,10 @@ namespace tt {
 namespace {
 
 constexpr int kShThreads = 256;
+// Thetas of the column level from here on take fp32 pairs: what fp32 drops
+// (terms below 2^-126 of the row's largest, 2^11 of them at most) is then less
+// than 2^-35 of theta.
+constexpr double kPairFloor = 8.271806125530277e-25;  // 2^-80
 
 // Column of the whole row scored by target row r (-1: a bonus row, or an
 // entry the decision reports as out of range): request b owns rows
@@ -48,11 +54,11 @@ __device__ int scored_column(const ShardArgs& a, int64_t r) {
 }
 
 // Each shard's own scored column of every target row; zeroes the row passes'
-// work counters and the error words.
-__global__ void shard_excl_kernel(ShardArgs a, int32_t* err) {
+// work counters. The row pass streams its first half beside it.
+__global__ void shard_excl_kernel(ShardArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i0 < int64_t(kWorkShards) * kWorkStride * a.S) a.work[i0] = 0ull;
-  if (i0 < 2) err[i0] = 0;
   for (int64_t r = i0; r < a.rows; r += int64_t(gridDim.x) * blockDim.x) {
     const int c = scored_column(a, r);
     for (int s = 0; s < a.S; ++s) {
@@ -64,6 +70,8 @@ __global__ void shard_excl_kernel(ShardArgs a, int32_t* err) {
 
 // One warp per (shard, row): the shard's record from its chunk partials.
 __global__ void shard_summary_kernel(ShardArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_dependency_wait();
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t stride = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -105,11 +113,15 @@ __device__ __forceinline__ double warp_scan_d(double v, int lane) {
 
 // One CTA per request: merge the gathered records of the request's m + 1
 // target rows (split-lse), accept test, residual or bonus draw.
+// Bound by its chain of dependent accesses and by fp64's rate: 27 us for 64
+// requests with a row per warp in the merge and the column level in fp64, 15 us
+// now (both cold).
 __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a) {
   constexpr int kWarps = kShThreads / 32;
   constexpr int kPer = kChunk / kShThreads;  // columns per thread in the fine level
   __shared__ float s_p[TT_MAX_M];
   __shared__ double s_wsum[kWarps];
+  __shared__ F2 s_wsum2[kWarps];
   __shared__ int s_acc, s_bad, s_shard, s_chunk, s_hit, s_last;
   __shared__ double s_theta, s_tterm;
   __shared__ float s_M;
@@ -130,6 +142,13 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
       if (c < 0 || c >= a.V) bad = 1;
     }
   if (__syncthreads_or(bad)) st |= TT_REQ_ID_OUT_OF_RANGE;
+  const uint64_t req = a.request_base + uint64_t(b);
+  float q0 = 0.f, u0 = 0.f;  // the thread's first draft token: q and its uniform
+  if (st == 0 && tid < m) {
+    q0 = a.q_hat[t0 + tid];
+    u0 = float(philox_uniform(a.seed, uint64_t(tid), 0, req));
+  }
+  grid_dependency_wait();  // (inputs only until here)
   if (st == 0 && a.err && a.err[0] == a.epoch) st = a.err[1];  // a row pass failed
   if (st != 0) {
     if (tid == 0) {
@@ -147,20 +166,32 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
   }
   __syncthreads();
   const ShardRec none = {-INFINITY, 0.f, 0.f, __int_as_float(0x7fffffff)};
-  // the merge: lane s holds shard s's record of the row
-  for (int j = warp; j <= m; j += kWarps) {
+  // The merge, four rows per warp: lane s of eight holds shard s's record of the
+  // row. (fp64 runs at two lanes a clock on an SM: a row per warp, with 24 lanes
+  // idle, made this the longest part of the kernel.)
+  constexpr int kRows = 32 / TT_MAX_SHARDS;
+  const int sl = lane % TT_MAX_SHARDS;
+  for (int j0 = warp * kRows; j0 <= m; j0 += kWarps * kRows) {
+    const int j = j0 + lane / TT_MAX_SHARDS;
     const int64_t row = int64_t(t0) + b + j;
-    const ShardRec R = lane < a.S ? a.rec[lane * a.rows + row] : none;
-    const float M = warp_max_f(fmaxf(R.m, R.st));  // fmaxf skips the NaN of a non-owner
+    const ShardRec R = j <= m && sl < a.S ? a.rec[sl * a.rows + row] : none;
+    float M = fmaxf(R.m, R.st);  // fmaxf skips the NaN of a non-owner
+#pragma unroll
+    for (int o = TT_MAX_SHARDS / 2; o > 0; o >>= 1)
+      M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     double z = 0.0, pt = 0.0;
     if (M > -INFINITY && M < INFINITY) {
       z = (double(R.s_hi) + double(R.s_lo)) * pow2_rel(R.m, M);
       pt = pow2_rel(R.st, M);
     }
-    z = warp_sum_d(z + pt);
-    pt = warp_sum_d(pt);  // the one owner's term
+    z += pt;
+#pragma unroll
+    for (int o = TT_MAX_SHARDS / 2; o > 0; o >>= 1) {
+      z += __shfl_xor_sync(0xffffffffu, z, o);
+      pt += __shfl_xor_sync(0xffffffffu, pt, o);  // the one owner's term
+    }
     const bool ok = M > -INFINITY && M < INFINITY && z > 0.0 && z < INFINITY;
-    if (lane == 0) {
+    if (sl == 0 && j <= m) {
       if (!ok) s_bad = 1;
       const float p = ok ? float(pt / z) : 0.f;
       if (j < m) {
@@ -180,10 +211,10 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
     return;
   }
   // accept while u_j q_j < p_j (u < 1 exactly)
-  const uint64_t req = a.request_base + uint64_t(b);
   for (int j = tid; j < m; j += kShThreads) {
-    const float u = float(philox_uniform(a.seed, uint64_t(j), 0, req));
-    if (!(u * a.q_hat[t0 + j] < s_p[j])) atomicMin(&s_acc, j);
+    const float u = j == tid ? u0 : float(philox_uniform(a.seed, uint64_t(j), 0, req));
+    const float q = j == tid ? q0 : a.q_hat[t0 + j];
+    if (!(u * q < s_p[j])) atomicMin(&s_acc, j);
   }
   __syncthreads();
   const int acc = s_acc;
@@ -270,37 +301,79 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
     const int xs = a.excl[sh * a.rows + row];
     const int c0 = chunk * kChunk + tid * kPer;
     const char* rp = d.data + row * d.stride_bytes;
-    double mine = 0.0;
-    double mx[kPer];
+    float z[kPer];
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int x = c0 + k;
-      double w = 0.0;
-      if (x < d.V) {
-        if (x == xs) {
-          w = tt;
-        } else {
-          const float z = d.dtype == TT_F32 ? load_logit<TT_F32>(rp, x) : load_logit<TT_BF16>(rp, x);
-          w = pow2_rel(z * a.scale, M);
-        }
-      }
-      mx[k] = w;
-      mine += w;
+      z[k] = x >= d.V ? -INFINITY
+                      : (d.dtype == TT_F32 ? load_logit<TT_F32>(rp, x) : load_logit<TT_BF16>(rp, x)) *
+                            a.scale;
     }
-    const double wi = warp_scan_d(mine, lane);
-    if (lane == 31) s_wsum[warp] = wi;
-    __syncthreads();
-    double off = 0.0;
-    for (int w = 0; w < warp; ++w) off += s_wsum[w];
-    double run = off + wi - mine;  // mass before this thread's first column
     int last = -1;
+    if (th2 >= kPairFloor && th2 < INFINITY) {
+      // The terms are fp32 values (2^f from the SFU, the exponent split exactly),
+      // so their prefix sums are taken in fp32 pairs; the hit is the first column
+      // whose running mass passes theta.
+      F2 mine = {0.f, 0.f}, next[kPer];
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      if (mx[k] > 0.0) {
-        if (th2 >= run && th2 < run + mx[k]) atomicMin(&s_hit, c0 + k);
-        last = c0 + k;
+      for (int k = 0; k < kPer; ++k) {
+        const int x = c0 + k;
+        F2 w = {0.f, 0.f};
+        if (x == xs && x < d.V) {
+          w.hi = float(tt);
+          w.lo = float(tt - double(w.hi));
+        } else if (z[k] > -INFINITY) {
+          w.hi = exp2_scaled(z[k], 1.f, M);
+        }
+        mine = f2_add(mine, w);
+        next[k] = mine;
+        if (w.hi > 0.f) last = x;
       }
-      run += mx[k];
+      F2 incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const F2 v = shfl_up_f2(incl, o);
+        if (lane >= o) incl = f2_add(v, incl);
+      }
+      if (lane == 31) s_wsum2[warp] = incl;
+      const F2 prev = shfl_up_f2(incl, 1);
+      __syncthreads();
+      F2 run = {0.f, 0.f};  // mass before this thread's first column
+      for (int w = 0; w < warp; ++w) run = f2_add(run, s_wsum2[w]);
+      if (lane > 0) run = f2_add(run, prev);
+      const float th = float(th2);
+      const F2 thp = {th, float(th2 - double(th))};
+      int hit = 0x7fffffff;
+#pragma unroll
+      for (int k = kPer - 1; k >= 0; --k)
+        if (f2_lt(thp, f2_add(run, next[k]))) hit = c0 + k;
+      hit = __reduce_min_sync(0xffffffffu, hit);
+      if (lane == 0 && hit != 0x7fffffff) atomicMin(&s_hit, hit);
+    } else {
+      // a theta so small that terms below fp32's range matter, or rounding past
+      // the end: fp64
+      double mine = 0.0;
+      double mx[kPer];
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int x = c0 + k;
+        mx[k] = x == xs && x < d.V ? tt : pow2_rel(z[k], M);
+        mine += mx[k];
+      }
+      const double wi = warp_scan_d(mine, lane);
+      if (lane == 31) s_wsum[warp] = wi;
+      __syncthreads();
+      double off = 0.0;
+      for (int w = 0; w < warp; ++w) off += s_wsum[w];
+      double run = off + wi - mine;  // mass before this thread's first column
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        if (mx[k] > 0.0) {
+          if (th2 >= run && th2 < run + mx[k]) atomicMin(&s_hit, c0 + k);
+          last = c0 + k;
+        }
+        run += mx[k];
+      }
     }
     if (last >= 0) atomicMax(&s_last, last);
     __syncthreads();
@@ -316,8 +389,6 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
 
 }  // namespace
 
-constexpr size_t kWorkBlockBytes = size_t(kWorkShards) * kWorkStride * sizeof(unsigned long long);
-
 ShardWorkspace shard_layout(void* base, int64_t rows, int S, const int32_t* nch) {
   ShardWorkspace w;
   char* p = static_cast<char*>(base);
@@ -332,16 +403,32 @@ ShardWorkspace shard_layout(void* base, int64_t rows, int S, const int32_t* nch)
                       : nullptr;
   w.excl = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * size_t(S) * rows));
   w.rec = reinterpret_cast<ShardRec*>(take(sizeof(ShardRec) * size_t(S) * rows));
-  w.work = reinterpret_cast<unsigned long long*>(take(kWorkBlockBytes * S));
+  w.work = reinterpret_cast<unsigned long long*>(take(kShardWorkBytes * S));
   w.err = reinterpret_cast<int32_t*>(take(2 * sizeof(int32_t)));
   w.bytes = off;
   return w;
 }
 
+// Launched while the grid before it drains (pdl): the kernels wait for it.
+template <typename Kern>
+static cudaError_t launch_after(Kern kernel, int blocks, int threads, const ShardArgs& args,
+                                cudaStream_t stream, bool pdl) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 cudaError_t launch_shard_excl(const ShardArgs& args, cudaStream_t stream) {
   const int64_t n = std::max<int64_t>(args.rows, int64_t(kWorkShards) * kWorkStride * args.S);
   const int blocks = int(std::min<int64_t>((n + 255) / 256, 4096));
-  shard_excl_kernel<<<blocks, 256, 0, stream>>>(args, const_cast<int32_t*>(args.err));
+  shard_excl_kernel<<<blocks, 256, 0, stream>>>(args);
   return cudaGetLastError();
 }
 
@@ -349,14 +436,12 @@ cudaError_t launch_shard_summary(const ShardArgs& args, cudaStream_t stream, int
   const int64_t warps = int64_t(args.S) * args.rows;
   if (warps == 0) return cudaSuccess;
   const int blocks = int(std::min<int64_t>((warps + 7) / 8, int64_t(sm_count) * 8));
-  shard_summary_kernel<<<blocks, 256, 0, stream>>>(args);
-  return cudaGetLastError();
+  return launch_after(shard_summary_kernel, blocks, 256, args, stream, true);
 }
 
-cudaError_t launch_decide_sharded(const ShardArgs& args, cudaStream_t stream) {
+cudaError_t launch_decide_sharded(const ShardArgs& args, cudaStream_t stream, bool pdl) {
   if (args.B == 0) return cudaSuccess;
-  decide_sharded_kernel<<<args.B, kShThreads, 0, stream>>>(args);
-  return cudaGetLastError();
+  return launch_after(decide_sharded_kernel, args.B, kShThreads, args, stream, pdl);
 }
 
 cudaError_t preload_shard() {

@@ -105,6 +105,21 @@ struct RowPassArgs {
   uint64_t wait_ns;          // limit of every pipeline wait (set by launch_rowpass: 2 s)
 };
 
+// The row pass over several column shards of the target rows at once.
+struct ShardRows {
+  const char* data;
+  int64_t stride_bytes, n_rows;
+  Partial* part;
+  const int32_t* excl;  // [target rows] the shard's own scored column or -1: read only
+                        // after the grid-dependency wait
+  int64_t end;          // row units of the shards up to this one
+  int V, col0, nch;
+};
+struct ShardPassArgs : RowPassArgs {  // (t: V of the whole row, scale; rows_t)
+  int S;
+  ShardRows sh[TT_MAX_SHARDS];
+};
+
 struct DecideArgs {
   int B, n_draft, n_target, max_k, max_m, full_q, mode_transfer_only;
   const int32_t* draft_off;
@@ -217,6 +232,9 @@ struct PrepArgs {
 size_t align_smem_per_pair(int max_k, int max_m, int tile_blocks);
 int align_tile_blocks(int max_k, int max_m, int window);
 cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream);
+// All shards of one type in one grid; `end` is filled in here.
+cudaError_t launch_shard_rowpass(const ShardPassArgs& args, int dt, cudaStream_t stream,
+                                 int sm_count, bool pdl);
 cudaError_t launch_rowpass(const RowPassArgs& args, int dt_d, int dt_t, cudaStream_t stream,
                            int sm_count, bool pdl);
 cudaError_t launch_decide(const DecideArgs& args, cudaStream_t stream, bool pdl);

@@ -7,10 +7,12 @@
 #include <cuda_runtime.h>
 
 #include "tt.h"
+#include "tt_device.cuh"
 
 namespace tt {
 
-struct Partial;
+// Work counters of one row pass.
+constexpr size_t kShardWorkBytes = size_t(kWorkShards) * kWorkStride * sizeof(unsigned long long);
 
 struct ShardDesc {
   const char* data;      // the shard's logits (device)
@@ -39,7 +41,7 @@ struct ShardArgs {
   ShardDesc sh[TT_MAX_SHARDS];
   int32_t* excl;             // [S * rows] scored column within each shard, or -1
   ShardRec* rec;             // [S * rows]
-  unsigned long long* work;  // S row-pass work counter blocks (zeroed by shard_excl_kernel)
+  unsigned long long* work;  // row-pass work counter blocks (zeroed by shard_excl_kernel)
   float scale;               // log2(e) / T_t
   const float* q_hat;
   uint64_t seed, request_base;
@@ -56,7 +58,7 @@ struct ShardWorkspace {
   Partial* part[TT_MAX_SHARDS];
   int32_t* excl;
   ShardRec* rec;
-  unsigned long long* work;  // S blocks of kWorkBlockBytes
+  unsigned long long* work;  // S blocks of kShardWorkBytes, one per row pass (of a type)
   int32_t* err;
   size_t bytes;
 };
@@ -65,7 +67,7 @@ struct ShardWorkspace {
 ShardWorkspace shard_layout(void* base, int64_t rows, int S, const int32_t* nch);
 cudaError_t launch_shard_excl(const ShardArgs& args, cudaStream_t stream);
 cudaError_t launch_shard_summary(const ShardArgs& args, cudaStream_t stream, int sm_count);
-cudaError_t launch_decide_sharded(const ShardArgs& args, cudaStream_t stream);
+cudaError_t launch_decide_sharded(const ShardArgs& args, cudaStream_t stream, bool pdl);
 
 cudaError_t preload_shard();
 
