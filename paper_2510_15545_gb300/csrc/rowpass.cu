@@ -46,14 +46,14 @@ struct Desc {
   int32_t req;    // the row's request when its family has a repetition penalty, else -1
 };
 
-// Stage s is always refilled for the same consumer warp (s mod kConsumerWarps),
-// so a warp never waits on a stage more than one phase ahead of it: an
-// mbarrier parity wait cannot tell phase n from phase n + 2.
 // The variant that takes column shards of the target rows: all shards of one
 // type in one grid, so that one ring fill and one tail serve them all. Four
 // shards of 64 requests (415 MB) took four passes of 23 us in turn, 68 us now.
 constexpr int kShards = 3;
 
+// Stage s is always refilled for the same consumer warp (s mod kConsumerWarps),
+// so a warp never waits on a stage more than one phase ahead of it: an
+// mbarrier parity wait cannot tell phase n from phase n + 2.
 constexpr int kCandCap = 128;   // top-k candidates of one unit a warp keeps in shared memory
 constexpr int kDirectCap = 32;  // vectors at or above tau1 taken directly (more: tau2)
 constexpr int kLevel2Cap = 64;  // vector maxima ranked by counting (more: radix search)
