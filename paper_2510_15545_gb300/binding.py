@@ -281,6 +281,9 @@ def _logits(t: Optional[torch.Tensor]) -> Optional[_Logits]:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        # (the handle alone: the Stream object of current_stream() costs 2.9 us a call)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -295,6 +298,13 @@ def _check(fn: str, code: int):
 
 def _empty(n, dtype, device):
     return torch.empty(max(int(n), 1), dtype=dtype, device=device)
+
+
+def _need(o, key, n, dtype, device):
+    """An output that the caller did not pass (an allocation for each one that
+    was passed, dropped at once, cost a repeated call 2 us apiece on the Grace host)."""
+    if key not in o:
+        o[key] = _empty(n, dtype, device)
 
 
 # ----------------------------------------------------------- entry points
@@ -323,11 +333,11 @@ class AlignCall:
                  out=None, stream=None):
         dev = batch.draft_off.device
         o = dict(out or {})
-        o.setdefault("path", _empty(2 * (batch.n_draft + batch.n_target), torch.int32, dev))
-        o.setdefault("path_len", _empty(batch.B, torch.int32, dev))
-        o.setdefault("cost", _empty(batch.B, torch.int32, dev))
-        o.setdefault("map", _empty(batch.n_target, torch.int32, dev))
-        o.setdefault("status", _empty(batch.B, torch.int32, dev))
+        _need(o, "path", 2 * (batch.n_draft + batch.n_target), torch.int32, dev)
+        _need(o, "path_len", batch.B, torch.int32, dev)
+        _need(o, "cost", batch.B, torch.int32, dev)
+        _need(o, "map", batch.n_target, torch.int32, dev)
+        _need(o, "status", batch.B, torch.int32, dev)
         self.out = o
         self._keep = [batch, vd, vt, o]
         self._b = batch._c()
@@ -355,8 +365,8 @@ def tt_transfer(batch: Batch, map: torch.Tensor, params: Params, *, draft_logits
                 draft_probs=None, ws=None, out=None, stream=None) -> dict:
     dev = batch.draft_off.device
     o = dict(out or {})
-    o.setdefault("q_hat", _empty(batch.n_target, torch.float32, dev))
-    o.setdefault("status", _empty(batch.B, torch.int32, dev))
+    _need(o, "q_hat", batch.n_target, torch.float32, dev)
+    _need(o, "status", batch.B, torch.int32, dev)
     if ws is None and draft_logits is not None:
         ws = workspace(batch, draft_logits.shape[1], 0, dev, params)
     keep = []
@@ -374,11 +384,11 @@ def tt_verify(batch: Batch, q_hat: torch.Tensor, target_logits: torch.Tensor, pa
               draft_logits=None, map=None, ws=None, out=None, stream=None) -> dict:
     dev = batch.target_off.device
     o = dict(out or {})
-    o.setdefault("accepted", _empty(batch.B, torch.int32, dev))
-    o.setdefault("next_token", _empty(batch.B, torch.int32, dev))
-    o.setdefault("status", _empty(batch.B, torch.int32, dev))
-    o.setdefault("p_hat", _empty(batch.n_target, torch.float32, dev))
-    o.setdefault("lse", _empty(batch.n_target + batch.B, torch.float32, dev))
+    _need(o, "accepted", batch.B, torch.int32, dev)
+    _need(o, "next_token", batch.B, torch.int32, dev)
+    _need(o, "status", batch.B, torch.int32, dev)
+    _need(o, "p_hat", batch.n_target, torch.float32, dev)
+    _need(o, "lse", batch.n_target + batch.B, torch.float32, dev)
     if ws is None:
         Vd = draft_logits.shape[1] if (params.full_q and draft_logits is not None) else 0
         ws = workspace(batch, Vd, target_logits.shape[1], dev, params)
@@ -424,15 +434,14 @@ def tt_verify_sharded(batch: Batch, q_hat: torch.Tensor, shards, params: Params,
     records [S, n_target + B, 4] (max, sum hi, sum lo, scored logit or NaN)."""
     dev = batch.target_off.device
     o = dict(out or {})
-    o.setdefault("accepted", _empty(batch.B, torch.int32, dev))
-    o.setdefault("next_token", _empty(batch.B, torch.int32, dev))
-    o.setdefault("status", _empty(batch.B, torch.int32, dev))
-    o.setdefault("p_hat", _empty(batch.n_target, torch.float32, dev))
-    o.setdefault("lse", _empty(batch.n_target + batch.B, torch.float32, dev))
+    _need(o, "accepted", batch.B, torch.int32, dev)
+    _need(o, "next_token", batch.B, torch.int32, dev)
+    _need(o, "status", batch.B, torch.int32, dev)
+    _need(o, "p_hat", batch.n_target, torch.float32, dev)
+    _need(o, "lse", batch.n_target + batch.B, torch.float32, dev)
     rows = batch.n_target + batch.B
-    if summaries:
-        o.setdefault("summaries", torch.empty((len(shards), rows, 4), dtype=torch.float32,
-                                              device=dev))
+    if summaries and "summaries" not in o:
+        o["summaries"] = torch.empty((len(shards), rows, 4), dtype=torch.float32, device=dev)
     sh, keep_sh = _shards(shards)
     L = load()
     if ws is None:
@@ -597,9 +606,9 @@ def tt_encode(draft_off: torch.Tensor, draft_ids: torch.Tensor, vd: VocabTable, 
     if capacity is None:
         capacity = B * int(max_m)
     o = dict(out or {})
-    o.setdefault("target_off", _empty(B + 1, torch.int32, dev))
-    o.setdefault("target_ids", _empty(capacity, torch.int32, dev))
-    o.setdefault("status", _empty(B, torch.int32, dev))
+    _need(o, "target_off", B + 1, torch.int32, dev)
+    _need(o, "target_ids", capacity, torch.int32, dev)
+    _need(o, "status", B, torch.int32, dev)
     if ws is None:
         ws = torch.empty(max(tt_encode_workspace_bytes(B, max_m), 256), dtype=torch.uint8,
                          device=dev)
