@@ -48,7 +48,7 @@ struct Desc {
 
 // The variant that takes column shards of the target rows: all shards of one
 // type in one grid, so that one ring fill and one tail serve them all. Four
-// shards of 64 requests (415 MB) took four passes of 23 us in turn, 68 us now.
+// shards of 64 requests (436 MB) took four passes of 23 us in turn, 68 us now.
 constexpr int kShards = 3;
 
 // Stage s is always refilled for the same consumer warp (s mod kConsumerWarps),
@@ -67,7 +67,7 @@ struct Ring {
   static constexpr bool kLists = SEL == 1 || SEL == 2;
   static constexpr size_t kScratch = kLists ? size_t(kConsumerWarps) * kCandCap * sizeof(Cand) : 0;
   static constexpr size_t kSmem =
-      size_t(kRingBytes) + kStages * (2 * sizeof(uint64_t) + sizeof(Desc)) + kScratch;
+      size_t(kRingBytes) + kStages * (3 * sizeof(uint64_t) + sizeof(Desc)) + kScratch;
   static_assert(kStages % kConsumerWarps == 0, "each stage belongs to one consumer warp");
   static constexpr int kGrabMin = kGrabMinBytes / kStageBytes > 0 ? kGrabMinBytes / kStageBytes : 1;
   static constexpr int kGrabMax = kGrabMaxBytes / kStageBytes;
@@ -148,30 +148,25 @@ __device__ __forceinline__ int req_lookup(const int32_t* off, int B, bool tgt, R
 }
 
 // Repetition penalty: where a unit's penalized columns lie, and the first 32
-// of them, one per lane. A consumer warp loads them for the unit that it will
-// most likely take next, kConsumerWarps further on in the row, while it works
-// on the current one: each is two dependent accesses, of a microsecond and more
-// beside the streaming row pass, which a warp would wait for on every unit.
+// of them, one per lane. A consumer warp loads them while the unit's copy is
+// still on its way: two dependent accesses, of a microsecond and more beside
+// the streaming row pass.
 struct PenUnit {
-  int64_t row;      // 2 * row + family; -1: none
-  int32_t unit;
   int32_t lo, hi;   // the unit's entries
   int32_t pos;      // the row's position in its request
   PenEntry e;       // this lane's entry (lo + lane); column -1: none
 };
 
-// First half: the unit's range of entries.
-__device__ __forceinline__ PenUnit pen_range(const RowPassArgs& a, const Desc& d, int unit) {
+__device__ __forceinline__ PenUnit pen_unit(const RowPassArgs& a, const Desc& d, int cps,
+                                            int lane) {
   const RowSet& S = d.set ? a.t : a.d;
-  const int64_t at = int64_t(d.req) * (S.nch + 1) + unit;
+  if (d.row < 0 || !S.pen || d.req < 0) return {0, 0, 0, {-1, 0}};
+  const int64_t at = int64_t(d.req) * (S.nch + 1) + d.chunk / cps;
   const int base = S.pbase[d.req];
   const int64_t first = d.set ? int64_t(a.target_off[d.req]) + d.req : a.draft_off[d.req];
-  return {d.row * 2 + d.set, unit, base + S.pstart[at], base + S.pstart[at + 1],
-          int32_t(d.row - first), {-1, 0}};
-}
-// Second half: its first entries.
-__device__ __forceinline__ void pen_entries(PenUnit& p, const RowSet& S, int lane) {
-  if (p.row >= 0 && p.lo + lane < p.hi) p.e = S.pen[p.lo + lane];
+  PenUnit p = {base + S.pstart[at], base + S.pstart[at + 1], int32_t(d.row - first), {-1, 0}};
+  if (p.lo + lane < p.hi) p.e = S.pen[p.lo + lane];
+  return p;
 }
 
 // Logit z penalized by theta (first position `first` of its column, row `pos`).
@@ -389,12 +384,40 @@ __device__ __forceinline__ Partial nuc_chunk_partial(const char* stage, const De
   return Partial{m, __fadd_rn(hs, ls)};
 }
 
+// The bar of a row (see select_unit), kept for one row of each family per CTA:
+// the row's index (there are fewer than 2^32) above an order-preserving key of
+// the value.
+__device__ __forceinline__ uint32_t bar_key(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float row_bar(const unsigned long long* seen, uint32_t row) {
+  const unsigned long long w = *reinterpret_cast<const volatile unsigned long long*>(seen);
+  const uint32_t k = uint32_t(w);
+  return uint32_t(w >> 32) == row
+             ? __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k)
+             : -INFINITY;
+}
+__device__ __forceinline__ void raise_bar(unsigned long long* seen, uint32_t row, float v) {
+  const unsigned long long w = (static_cast<unsigned long long>(row) << 32) | bar_key(v);
+  // (another row's bar is replaced; a race between rows costs a bar, not a result)
+  if (uint32_t(*reinterpret_cast<volatile unsigned long long*>(seen) >> 32) == row)
+    atomicMax(seen, w);
+  else
+    *reinterpret_cast<volatile unsigned long long*>(seen) = w;
+}
+
 // One consumer warp writes the top-K (value, column) list of one unit held in
 // shared memory (its whole 16-byte vectors) plus a ragged tail of fewer than
 // 16 bytes read directly, ordered by cand_before, padded with (-inf, -1);
 // columns are absolute. Each lane owns 16 vectors and keeps their maxima in
 // registers. A threshold at or below the unit's K-th largest element bounds
 // the candidates:
+//   The row's bar, the best K-th largest element of its units that this CTA has
+//   finished: nothing below it can be in the row's top-k, so that when at most
+//   32 vectors reach it their elements are the candidates, fewer than K often,
+//   and the sorts below are not needed (256 requests, bf16, top-20: 474 -> 465
+//   us a step).
 //   tau1, the K-th largest of the 64 values formed by each lane's two largest
 //   vector maxima (two bitonic sorts and a merge; K <= 32); K vectors reach
 //   it, so K elements do. Usually about K vectors reach tau1 and their
@@ -407,9 +430,12 @@ __device__ __forceinline__ Partial nuc_chunk_partial(const char* stage, const De
 // kCandCap (runs of equal logits) take K rounds of a warp-wide extraction over
 // the same vectors instead. The work per unit is thus nearly the same for
 // every unit, which keeps the stage ring from waiting on one slow warp.
-template <int DT>
+// release() gives the stage back as soon as its candidates are in the scratch, so
+// that the next copy runs beside the ranking (465 -> 453 us).
+template <int DT, typename Release>
 __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, int lane, int K,
-                            Cand* scratch, Cand* out, uint32_t tail_pen = 0u) {
+                            Cand* scratch, Cand* out, unsigned long long* seen, uint32_t tail_pen,
+                            Release&& release) {
   constexpr int VEC = DT == TT_F32 ? 4 : 8;  // logits per 16-byte vector
   constexpr int NV = kChunk * 4 / (16 * 32);   // vectors per lane in one stage
   constexpr uint32_t kTailBit = 1u << NV;      // flag of the lane's tail element
@@ -445,13 +471,20 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
     for (int v = 0; v < NV; ++v) f |= vm[v] >= t ? (1u << v) : 0u;
     return f & valid;
   };
-  // the 32 largest of the 64: half-cleaner of (m1 descending, m2 ascending)
-  const float top = warp_merge_desc(fmaxf(warp_sort<true>(m1, lane), warp_sort<false>(m2, lane)),
-                                    lane);
-  float tau = __shfl_sync(0xffffffffu, top, K - 1);
-  uint32_t flags = at_or_above(tau);
-  const int nf = __popc(flags);
-  const int F1 = int(__reduce_add_sync(0xffffffffu, unsigned(nf)));
+  const float bar = __shfl_sync(0xffffffffu, row_bar(seen, uint32_t(d.row)), 0);
+  float tau = bar;
+  uint32_t flags = at_or_above(bar);
+  int nf = __popc(flags);
+  int F1 = bar > -INFINITY ? int(__reduce_add_sync(0xffffffffu, unsigned(nf))) : kDirectCap + 1;
+  if (F1 > kDirectCap) {
+    // the 32 largest of the 64: half-cleaner of (m1 descending, m2 ascending)
+    const float top = warp_merge_desc(
+        fmaxf(warp_sort<true>(m1, lane), warp_sort<false>(m2, lane)), lane);
+    tau = __shfl_sync(0xffffffffu, top, K - 1);
+    flags = at_or_above(tau);
+    nf = __popc(flags);
+    F1 = int(__reduce_add_sync(0xffffffffu, unsigned(nf)));
+  }
   if (F1 > kDirectCap) {
     // tau2: the K-th largest maximum; every vector that reaches it reaches tau1
     if (F1 <= kLevel2Cap) {
@@ -535,6 +568,7 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
       }
     }
     __syncwarp();
+    release();
     for (int i = lane; i < C; i += 32) {
       const Cand ci = scratch[i];
       int r = 0;
@@ -544,6 +578,7 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
         r += cand_before(cj.v, cj.c, ci.v, ci.c);
       }
       if (r < K) out[r] = Cand{ci.v, col0 + ci.c};
+      if (r == K - 1) raise_bar(seen, uint32_t(d.row), ci.v);
     }
     for (int r = C + lane; r < K; r += 32) out[r] = Cand{-INFINITY, -1};
   } else {
@@ -589,6 +624,8 @@ __device__ void select_unit(const char* stage, const Desc& d, const RowView& S, 
         pc = 0x7fffffff;
       }
     }
+    __syncwarp();
+    release();
   }
   __syncwarp();  // the scratch is free for the next unit
 }
@@ -604,15 +641,21 @@ __global__ void __launch_bounds__(kThreads, 3)
   char* stages = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRingBytes);
   uint64_t* empty = full + R::kStages;
-  Desc* desc = reinterpret_cast<Desc*>(empty + R::kStages);
+  uint64_t* posted = empty + R::kStages;  // the stage's description is written
+  Desc* desc = reinterpret_cast<Desc*>(posted + R::kStages);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // a consumer warp's candidate scratch (filtered rows only)
   Cand* scratch = reinterpret_cast<Cand*>(desc + R::kStages) + (R::kLists ? warp * kCandCap : 0);
 
+  __shared__ unsigned long long seen[2];  // the last row's bar, per family
+  // penalized rows: consumers look at a stage's description before its data
+  const bool penalties = SEL == 2 && (a.d.pen || a.t.pen);
   if (threadIdx.x == 0) {
+    seen[0] = seen[1] = ~0ull;  // (no row)
     for (int s = 0; s < R::kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
+      mbar_init(&posted[s], 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -714,6 +757,7 @@ __global__ void __launch_bounds__(kThreads, 3)
           d.n_smem = 0;
         }
         desc[s] = d;
+        if (penalties) mbar_arrive(&posted[s]);
         if (copy_ok && bytes > 0) {
           mbar_arrive_expect_tx(&full[s], bytes);
           bulk_copy_g2s(stages + size_t(s) * R::kStageBytes, src, bytes, &full[s]);
@@ -811,6 +855,7 @@ __global__ void __launch_bounds__(kThreads, 3)
           break;
         }
         desc[s].row = -1;
+        if (penalties) mbar_arrive(&posted[s]);
         mbar_arrive(&full[s]);
         ++it;
       }
@@ -822,10 +867,19 @@ __global__ void __launch_bounds__(kThreads, 3)
   // (one thread's launch_dependents counts for its whole CTA: only the
   // producer lane gives it, after its grid-dependency wait, because the next
   // grid reads the alignment's outputs before its own wait)
-  PenUnit pu = {-1, 0, 0, 0, 0, {-1, 0}};  // the unit expected next (penalized rows)
   for (int it = warp;; it += kConsumerWarps) {
     const int s = it % R::kStages;
     const uint32_t par = (it / R::kStages) & 1;
+    PenUnit pu;
+    if constexpr (SEL == 2) {
+      if (penalties) {
+        if (!mbar_wait(&posted[s], par, a.wait_ns)) {
+          if (lane == 0) report_error(a.err, a.epoch, TT_REQ_TIMEOUT);
+          break;
+        }
+        pu = pen_unit(a, desc[s], desc[s].set ? R::kCpsT : R::kCpsD, lane);
+      }
+    }
     if (!mbar_wait(&full[s], par, a.wait_ns)) {
       if (lane == 0) report_error(a.err, a.epoch, TT_REQ_TIMEOUT);
       break;
@@ -861,27 +915,24 @@ __global__ void __launch_bounds__(kThreads, 3)
       if constexpr (SEL == 2) {
         if (S.pen && d.req >= 0) {
           char* wstage = stages + size_t(s) * R::kStageBytes;
-          const int unit = d.chunk / cps;
-          if (pu.row != d.row * 2 + d.set || pu.unit != unit) {
-            pu = pen_range(a, d, unit);
-            pen_entries(pu, S, lane);
-          }
           tail_pen = (d.set ? DTT : DTD) == TT_F32 ? apply_penalty<TT_F32>(wstage, d, S, pu, lane)
                                                    : apply_penalty<TT_BF16>(wstage, d, S, pu, lane);
-          pu.row = -1;
-          if (unit + kConsumerWarps < S.nlist) pu = pen_range(a, d, unit + kConsumerWarps);
         }
       }
+      auto release = [&]() {
+        if (lane == 0 && !(blockIdx.x == 0 && it == a.stall_stage))
+          mbar_arrive(&empty[s]);  // the stage's bytes are consumed
+      };
       if constexpr (DTD == DTT) {
-        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
+        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, &seen[d.set], tail_pen,
+                         release);
       } else if (d.set) {
-        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
+        select_unit<DTT>(stage, d, V, lane, S.top_k, scratch, out, &seen[d.set], tail_pen,
+                         release);
       } else {
-        select_unit<DTD>(stage, d, V, lane, S.top_k, scratch, out, tail_pen);
+        select_unit<DTD>(stage, d, V, lane, S.top_k, scratch, out, &seen[d.set], tail_pen,
+                         release);
       }
-      if (SEL == 2 && S.pen && d.req >= 0) pen_entries(pu, S, lane);
-      if (lane == 0 && !(blockIdx.x == 0 && it == a.stall_stage))
-        mbar_arrive(&empty[s]);  // the stage's bytes are consumed
       continue;
     }
     // the unit's chunks (two for bf16 rows), each reduced on its own by one

@@ -52,7 +52,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 }
 // Bulk copy of a piece of a streamed row. Rows are read once each: their lines
 // leave L2 first, and what is read again (partials, lists, tables, offsets)
-// stays: 64 requests (440 MB) 86.9 -> 84.5 us, filtered and sharded ones 3 % less,
+// stays: 64 requests (500 MB) 86.9 -> 84.5 us, filtered and sharded ones 3 % less,
 // batches of GBs the same. (The policy is formed at each copy: held in
 // registers, it took the row pass past what lets a decision CTA sit beside it,
 // 96 us.)
