@@ -465,7 +465,13 @@ __global__ void __launch_bounds__(kConsThreads) consistency_kernel(ConsArgs a) {
 
 // --------------------------------------------------- delta-pos histogram
 
-constexpr int kDposWarps = 4;
+// Two CTAs per SM at most, as each adds its bins to the global ones; a request
+// is a chain of three dependent accesses, so a CTA has sixteen warps where four
+// would have to take several requests in turn (4096 requests of 64 tokens: 10.6
+// us with four warps, 5.0 with sixteen; 32 requests: 6.0 with either, and 0.6 us
+// less around it with four).
+constexpr int kDposWarps = 4, kDposWarpsMany = 16;
+constexpr int kDposFly = 4;  // entries in flight per lane
 
 struct DposArgs {
   int B, n_draft, n_target, mode, n_bins;
@@ -477,13 +483,13 @@ struct DposArgs {
   unsigned long long* hist;
 };
 
-__global__ void __launch_bounds__(32 * kDposWarps) dpos_kernel(DposArgs a) {
+__global__ void __launch_bounds__(32 * kDposWarpsMany) dpos_kernel(DposArgs a) {
   __shared__ unsigned int s_hist[TT_MAX_DPOS_BINS];
   for (int x = threadIdx.x; x < a.n_bins; x += blockDim.x) s_hist[x] = 0;
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int top = a.n_bins - 1;
-  for (int b = blockIdx.x * kDposWarps + warp; b < a.B; b += gridDim.x * kDposWarps) {
+  for (int b = blockIdx.x * warps + warp; b < a.B; b += gridDim.x * warps) {
     if (!csr_ok(a.draft_off, b, a.n_draft) || !csr_ok(a.target_off, b, a.n_target)) continue;
     const int d0 = a.draft_off[b], k = a.draft_off[b + 1] - d0;
     const int t0 = a.target_off[b], m = a.target_off[b + 1] - t0;
@@ -491,9 +497,16 @@ __global__ void __launch_bounds__(32 * kDposWarps) dpos_kernel(DposArgs a) {
     if (len <= 0) continue;
     if (a.mode == 0) {
       const int32_t* pp = a.path + 2 * (int64_t(d0) + t0);
-      for (int x = lane; x < len; x += 32) {
-        const int d = abs(pp[2 * x] - pp[2 * x + 1]);
-        atomicAdd(&s_hist[min(d, top)], 1u);
+      for (int x0 = lane; x0 < len; x0 += 32 * kDposFly) {
+        int d[kDposFly];
+#pragma unroll
+        for (int q = 0; q < kDposFly; ++q) {
+          const int x = x0 + 32 * q;
+          d[q] = x < len ? abs(pp[2 * x] - pp[2 * x + 1]) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < kDposFly; ++q)
+          if (x0 + 32 * q < len) atomicAdd(&s_hist[min(d[q], top)], 1u);
       }
     } else {
       for (int j = lane; j < m; j += 32) {
@@ -699,10 +712,11 @@ extern "C" tt_status tt_dpos_hist(const tt_batch* batch, const int32_t* path,
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int want = (a.B + kDposWarps - 1) / kDposWarps;
+  const int warps = a.B > 2 * sms * kDposWarps ? kDposWarpsMany : kDposWarps;
+  const int want = (a.B + warps - 1) / warps;
   const int grid = want < 2 * sms ? want : 2 * sms;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  dpos_kernel<<<grid, 32 * kDposWarps, 0, s>>>(a);
+  dpos_kernel<<<grid, 32 * warps, 0, s>>>(a);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? TT_OK : record_cuda_error(e);
 }

@@ -2,7 +2,8 @@
 the oracle: batches at the edges of the blocks that one CTA of the compaction
 takes, capacities that cut at a block's edge or inside one, texts around the
 threads of a CTA and at the byte limit, drafts of more tokens than threads,
-tokens around eight bytes (where the index's keys change), crowded tables."""
+tokens around eight bytes (where the index's keys change); and the delta-pos
+histogram around its launch shapes."""
 import numpy as np
 import pytest
 import torch
@@ -84,3 +85,21 @@ def test_consistency_sizes(k, m):
     o = oracle.consistency(d_off, d_ids, t_off, t_ids, vd.blob, vd.off, vt.blob, vt.off, 256, 512)
     assert np.array_equal(g, o)
     assert list(o) == [0, oracle.ST_INCONSISTENT, oracle.ST_ID_RANGE]
+
+
+@pytest.mark.parametrize("B", [1, 4, 5, 1216, 1217, 5000])
+def test_dpos_hist_batches(B):
+    """Batches around the CTA's warps and around the size where CTAs grow; paths
+    around the entries a warp has in flight."""
+    rng = np.random.default_rng(B)
+    k, m = rng.integers(1, 80, B), rng.integers(1, 80, B)
+    d_off = np.concatenate([[0], np.cumsum(k)]).astype(np.int32)
+    t_off = np.concatenate([[0], np.cumsum(m)]).astype(np.int32)
+    lens = np.minimum(k + m, rng.choice([0, 1, 31, 32, 33, 127, 128, 129, 160], B)).astype(np.int32)
+    path = rng.integers(0, 90, 2 * (int(d_off[-1]) + int(t_off[-1]))).astype(np.int32)
+    mp = rng.integers(0, 80, int(t_off[-1])).astype(np.int32)
+    batch = tt.Batch.from_host(d_off, np.zeros(int(d_off[-1])), t_off, np.zeros(int(t_off[-1])))
+    dev = [torch.as_tensor(x, device="cuda") for x in (path, lens, mp)]
+    for mode in (0, 1):
+        g = tt.tt_dpos_hist(batch, *dev, mode, 40).cpu().numpy()
+        assert np.array_equal(g, oracle.dpos_hist(d_off, t_off, path, lens, mp, mode, 40))
