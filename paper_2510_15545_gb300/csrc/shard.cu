@@ -54,8 +54,16 @@ __device__ int scored_column(const ShardArgs& a, int64_t r) {
 }
 
 // Each shard's own scored column of every target row; zeroes the row passes'
-// work counters. The row pass streams its first half beside it.
-__global__ void shard_excl_kernel(ShardArgs a) {
+// work counters and the error words. The row pass streams its first half beside
+// it; the error words, which that half may write, are zeroed before it starts.
+__global__ void shard_excl_kernel(ShardArgs a, int32_t* err) {
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < 2) {
+      err[threadIdx.x] = 0;
+      __threadfence();
+    }
+    __syncthreads();
+  }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t i0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i0 < int64_t(kWorkShards) * kWorkStride * a.S) a.work[i0] = 0ull;
@@ -428,7 +436,7 @@ static cudaError_t launch_after(Kern kernel, int blocks, int threads, const Shar
 cudaError_t launch_shard_excl(const ShardArgs& args, cudaStream_t stream) {
   const int64_t n = std::max<int64_t>(args.rows, int64_t(kWorkShards) * kWorkStride * args.S);
   const int blocks = int(std::min<int64_t>((n + 255) / 256, 4096));
-  shard_excl_kernel<<<blocks, 256, 0, stream>>>(args);
+  shard_excl_kernel<<<blocks, 256, 0, stream>>>(args, const_cast<int32_t*>(args.err));
   return cudaGetLastError();
 }
 
