@@ -835,9 +835,10 @@ cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream) {
     n_sm[dev] = 148;
   AlignArgs a = args;
   const int64_t sms = n_sm[dev];
-  // Large pairs: a CTA per pair, of kAlignMid warps, or of kAlignWide warps where one such CTA per pair would leave the chip idle (at
-  // most two pairs per SM) and for drafts whose sweep needs four row pairs per
-  // lane. Before the row pass as many CTAs as kAlignRoom holds per SM, which
+  // Large pairs: a CTA per pair, of kAlignMid warps, or of kAlignWide warps
+  // where one such CTA per pair would leave the chip idle (at most two pairs
+  // per SM) and for drafts whose sweep needs four row pairs per lane. Before
+  // the row pass as many CTAs as kAlignRoom holds per SM, which
   // loop over the pairs.
   if (a.tile_blocks >= 128) {
     a.pairs_per_block = 1;

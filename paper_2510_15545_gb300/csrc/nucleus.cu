@@ -670,9 +670,12 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
     unsigned long long tot = lane < nch ? sm.cacc[lane] : 0ull;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    const KeptNorm kn = kept_norm(tot, M);
-    if (lane < nch) um[lane] = __ull2float_rn(sm.cacc[lane]) * kn.inv_tot;
-    if (lane == 0) *head = KeptHead{kn.lse, 1, tau, tau_col, M, kn.inv_s};
+    const KeptNorm kn = kept_norm(tot);
+    if (lane < nch) um[lane] = kept_share(sm.cacc[lane], kn);
+    if (lane == 0) {
+      const KeptScale ks = kept_scale(kn, M);
+      *head = KeptHead{ks.lse, 1, tau, tau_col, M, ks.inv_s};
+    }
     __syncwarp();  // shared memory is reused by the warp's next row
   }
 }
@@ -975,9 +978,12 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
     unsigned long long tot = 0ull;
     for (int c = tid; c < nch; c += kNT) tot += sm.cacc[c];
     tot = block_sum_u64(tot, sm, lane, warp);
-    const KeptNorm kn = kept_norm(tot, M);
-    for (int c = tid; c < nch; c += kNT) um[c] = __ull2float_rn(sm.cacc[c]) * kn.inv_tot;
-    if (tid == 0) *head = KeptHead{kn.lse, tot > 0ull ? 1 : 0, tau, tau_col, M, kn.inv_s};
+    const KeptNorm kn = kept_norm(tot);
+    for (int c = tid; c < nch; c += kNT) um[c] = kept_share(sm.cacc[c], kn);
+    if (tid == 0) {
+      const KeptScale ks = kept_scale(kn, M);
+      *head = KeptHead{ks.lse, tot > 0ull ? 1 : 0, tau, tau_col, M, ks.inv_s};
+    }
     __syncthreads();  // shared memory is reused by the next row
   }
   }

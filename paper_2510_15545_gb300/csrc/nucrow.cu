@@ -705,9 +705,12 @@ __device__ void cut_rows(const NucRowArgs& a, NrSmem& sm, int tid) {
           for (int c = lane; c < nch; c += 32) tot += sm.u.cacc[c];
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-          const KeptNorm kn = kept_norm(tot, M);
-          for (int c = tid; c < nch; c += kCT) um[c] = __ull2float_rn(sm.u.cacc[c]) * kn.inv_tot;
-          if (tid == 0) *head = KeptHead{kn.lse, 1, tau, tau_col, M, kn.inv_s};
+          const KeptNorm kn = kept_norm(tot);
+          for (int c = tid; c < nch; c += kCT) um[c] = kept_share(sm.u.cacc[c], kn);
+          if (tid == 0) {
+            const KeptScale ks = kept_scale(kn, M);
+            *head = KeptHead{ks.lse, 1, tau, tau_col, M, ks.inv_s};
+          }
           settled = true;
         }
       }

@@ -53,24 +53,61 @@ __device__ __forceinline__ float exp2_scaled(float z, float scale, float M) {
   return ex2_approx(f) * __int_as_float((int(n) + 127) << 23);
 }
 
-// The normaliser of a nucleus row from its kept mass `tot` (40-bit fixed point,
-// relative to 2^M): 2^40 / tot and the natural log of tot 2^(M - 40), from fp32
-// pairs (about an ulp; fp64 is slow here). Every kernel that settles nucleus
-// rows forms them this way, so that a row's result does not depend on which did.
+// The kept set of a nucleus row from its kept mass `tot` (40-bit fixed point,
+// relative to 2^M). Every kernel that settles nucleus rows forms these the same
+// way, so that a row's result does not depend on which did.
 constexpr float kFixScale = 1099511627776.f;  // 2^40
+// A chunk's share c / tot of it, from fp32 pairs (about half an ulp; a division
+// in fp64, which is slow here, for each chunk of every row held the cuts up).
 struct KeptNorm {
-  float inv_tot, inv_s, lse;  // 1 / tot, 2^40 / tot
+  float hi, lo, inv;  // tot = hi + lo; 1 / tot
 };
-__device__ __forceinline__ KeptNorm kept_norm(unsigned long long tot, float M) {
-  const float sh = __ull2float_rn(tot);
-  const float sl = __ll2float_rn((long long)(tot - __float2ull_rn(sh)));
-  const float r = __frcp_rn(sh);
-  const float inv = fmaf(r, fmaf(-sl, r, fmaf(-sh, r, 1.f)), r);
-  const F2 l2 = two_sum(M, log2f(sh * (1.f / kFixScale)));
-  const float ln2 = 0.693147180559945f, ln2l = 1.904654299957768e-9f;
+__device__ __forceinline__ KeptNorm kept_norm(unsigned long long tot) {
+  const float hi = __ull2float_rn(tot);
+  const float lo = __ll2float_rn((long long)(tot - __float2ull_rn(hi)));
+  const float r = __frcp_rn(hi);
+  return {hi, lo, fmaf(r, fmaf(-lo, r, fmaf(-hi, r, 1.f)), r)};
+}
+__device__ __forceinline__ float kept_share(unsigned long long c, const KeptNorm& k) {
+  const float hi = __ull2float_rn(c);
+  const float lo = __ll2float_rn((long long)(c - __float2ull_rn(hi)));
+  const float q = __fmul_rn(hi, k.inv);
+  return fmaf(__fadd_rn(fmaf(-q, k.hi, hi), fmaf(-q, k.lo, lo)), k.inv, q);
+}
+// The natural log of the normaliser sum, and 2^40 / tot. log(m 2^e) = e log 2 +
+// 2 atanh((m - 1) / (m + 1)), m in [0.7, 1.42), by atanh's series in s <= 0.172,
+// whose first term and the sum are held in pairs: the result is rounded once,
+// give or take 1e-9. (fp64 here, by one thread per row, made a step of 1024
+// requests 4 % slower; log2f added an ulp.)
+struct KeptScale {
+  float lse, inv_s;
+};
+__device__ __forceinline__ KeptScale kept_scale(const KeptNorm& k, float M) {
+  if (!(k.hi > 0.f)) return {-INFINITY, INFINITY};
+  int e = (__float_as_int(k.hi) >> 23) - 127;
+  float sc = __int_as_float((127 - e) << 23);  // 2^-e (tot < 2^64)
+  if (k.hi * sc > 1.41421356f) {
+    sc *= 0.5f;
+    ++e;
+  }
+  const float mh = k.hi * sc, ml = k.lo * sc;
+  const F2 num = two_sum(mh - 1.f, ml);  // (mh - 1 is exact)
+  F2 den = two_sum(mh, 1.f);
+  den.lo += ml;
+  const float s0 = __fdiv_rn(num.hi, den.hi);
+  const float s1 = __fdividef(fmaf(-s0, den.hi, num.hi) + fmaf(-s0, den.lo, num.lo), den.hi);
+  const float x = s0 * s0;
+  float P = fmaf(x, 1.f / 13.f, 1.f / 11.f);
+  P = fmaf(x, P, 1.f / 9.f);
+  P = fmaf(x, P, 1.f / 7.f);
+  P = fmaf(x, P, 1.f / 5.f);
+  P = fmaf(x, P, 1.f / 3.f) * x;
+  const float ln2 = 0.693147180559945f, ln2l = -1.904654299957768e-9f;
+  const F2 l2 = two_sum(M, float(e - 40));
   const float ph = __fmul_rn(l2.hi, ln2);
   const float pl = fmaf(l2.hi, ln2, -ph) + fmaf(l2.hi, ln2l, l2.lo * ln2);
-  return {inv, inv * kFixScale, ph + pl};
+  const F2 t = two_sum(ph, 2.f * s0);
+  return {t.hi + (t.lo + (pl + 2.f * fmaf(s0, P, s1))), k.inv * kFixScale};
 }
 
 __device__ __forceinline__ void grid_dependency_wait() {
