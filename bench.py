@@ -609,8 +609,8 @@ def run_mine(args):
         "dtw": {"ms_alone": align_alone_ms, "ms_in_step": align_ms,
                 "pairs_per_s_in_step": wl.B / (align_ms / 1e3),
                 "band_cells": cells, "band_cells_per_s": cells / (align_alone_ms / 1e3),
-                "note": "dtw_pairs_per_s: tt_align alone (one warp per pair), 200 calls; in "
-                        "the step the alignment takes one CTA per SM beside the row pass"},
+                "note": "dtw_pairs_per_s: tt_align alone (as many CTAs as fit), "
+                        "200 calls; in the step fewer run, beside the row pass"},
         "stage_ms": st,
         "roofline": {"bound": "hbm", "kernel": "rowpass_kernel", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak,
@@ -660,8 +660,9 @@ def _time_calls(fn, stream, n, warm=3):
 def run_align_alone(tt, wl, inp, prm, dev, stream):
     """tt_align on its own (DTW and the map i*(j), nothing after it), timed with
     CUDA events over repeated calls outside the step's timed region. Alone it
-    takes one warp per pair and as many CTAs as fit; inside tt_step the same
-    kernel runs on one CTA per SM so that the row pass streams beside it."""
+    takes as many CTAs as fit (a warp per pair, or several for large pairs);
+    inside tt_step fewer CTAs loop over the pairs so that the row pass streams
+    beside them."""
     call = tt.AlignCall(inp["batch"], inp["vd"], inp["vt"], prm, stream=stream)
     return _time_calls(call, stream, 200)
 
