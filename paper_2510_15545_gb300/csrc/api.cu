@@ -525,7 +525,9 @@ tt_status tt_transfer(const tt_batch* batch, const int32_t* map, const tt_logits
     r.pre_eighths = 4;
     d.err = ws.err;
     d.epoch = r.epoch;
-    // (the absent family's type is a placeholder: the draft's, one kernel variant)
+    // (the absent family's type is a placeholder: the draft's, one kernel variant.
+    // The penalty's sets may still be built when the row pass starts: it takes
+    // draft rows, and with them the sets, only after its grid-dependency wait.)
     if ((e = launch_rows(r, prm, ws, draft->dtype, draft->dtype, s, true)) != cudaSuccess)
       return cuda_fail(e);
   }
