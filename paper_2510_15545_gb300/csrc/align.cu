@@ -775,12 +775,18 @@ __global__ void __launch_bounds__(align_threads(WPP), 1024 / align_threads(WPP))
 
 }  // namespace
 
+// The band's half-width as the kernel takes it. |i - j| of a pair is below
+// TT_MAX_K + TT_MAX_M, so wider bands (any w >= 0 is allowed) are that band, and
+// the kernel's and the tile's arithmetic on twice the width fits an int.
+int align_window(int window) { return min(window, TT_MAX_K + TT_MAX_M); }
+
 // Blocks of the cost tile that a pair of k <= max_k and m <= max_m tokens can
 // need: (k + 1) / 2 row pairs of row_blocks(m, W0), W0 = max(window, |k - m|).
 // For a given k, the row grows with m while m >= k (so m = max_m is the
 // longest there); for m < k, 2 (k - m) + 2 falls while m grows, so a row has
 // at most max(2 window, 2 k / 3) + 4 band columns, and never more than k.
 int align_tile_blocks(int max_k, int max_m, int window) {
+  window = align_window(window);
   int most = 0;
   for (int k = 1; k <= max_k; ++k) {
     int w;

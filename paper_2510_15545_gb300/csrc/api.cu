@@ -344,14 +344,14 @@ tt_status fill_align_args(const tt_batch* bt, const tt_vocab* vd, const tt_vocab
   a.n_target = bt->n_target;
   a.max_k = bt->max_k;
   a.max_m = bt->max_m;
-  a.window = prm->window;
+  a.window = align_window(prm->window);
   a.draft_off = bt->draft_off;
   a.draft_ids = bt->draft_ids;
   a.target_off = bt->target_off;
   a.target_ids = bt->target_ids;
   a.vd = *vd;
   a.vt = *vt;
-  a.tile_blocks = align_tile_blocks(bt->max_k, bt->max_m, prm->window);
+  a.tile_blocks = align_tile_blocks(bt->max_k, bt->max_m, a.window);
   a.smem_per_pair = align_smem_per_pair(bt->max_k, bt->max_m, a.tile_blocks);
   if (a.smem_per_pair > size_t(kAlignSmemMax)) return TT_ERR_UNSUPPORTED;
   return TT_OK;

@@ -230,6 +230,7 @@ struct PrepArgs {
 };
 
 size_t align_smem_per_pair(int max_k, int max_m, int tile_blocks);
+int align_window(int window);
 int align_tile_blocks(int max_k, int max_m, int window);
 cudaError_t launch_align(const AlignArgs& args, cudaStream_t stream);
 // All shards of one type in one grid; `end` is filled in here.

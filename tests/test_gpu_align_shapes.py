@@ -75,3 +75,7 @@ def test_costs_past_16_bits():
     # and below 127 (the largest that the tile stores)
     _check([100, 33], [90, 100], 200, np.arange(97, 117), (8, -1), 3, n_vocab=40, min_len=100)
     _check([130], [140], 100, np.arange(97, 117), (8,), 4, n_vocab=40, min_len=60)
+
+
+def test_bands_wider_than_any_pair():
+    _check([3, 64, 200], [5, 90, 300], 8, np.arange(97, 117), (767, 768, 2**30, 2**31 - 1), 9)

@@ -193,3 +193,26 @@ def test_workspace_of_filter_families(lib):
     assert topk - plain >= lists
     assert plain < nuc < plain + rows * (units * 4 + 64) + 8 * 256
     assert nuc < topk
+
+
+def test_alignment_tile_holds_every_band(lib):
+    """Host sizing of the alignment's cost tile: at least what the kernel takes
+    of it for any pair (a row pair's columns within max(w, |k - m|), as 8-diagonal
+    blocks, an odd number), for every half-width an int holds. A half-width of
+    2^30 and more overflowed, and the tile was too small for the band."""
+    blocks = lib._ZN2tt17align_tile_blocksEiii
+    widths = (0, 1, 8, 255, 767, 768, 769, 2**30 - 1, 2**30, 2**31 - 2, 2**31 - 1)
+
+    def row_blocks(m, w0):
+        return ((min(2 * w0 + 2, m) + 15) >> 3) | 1
+
+    for max_k, max_m in [(1, 1), (5, 9), (64, 81), (256, 512), (256, 1)]:
+        whole = blocks(max_k, max_m, -1)
+        for w in widths:
+            need = max((k + 1) // 2 * row_blocks(m, max(w, abs(k - m)))
+                       for k in {1, max_k // 3, max_k // 2, max_k - 1, max_k} - {0}
+                       for m in {1, max_m // 3, max_m // 2, max_m - 1, max_m} - {0})
+            assert need <= blocks(max_k, max_m, w) <= whole + (max_k + 1), (max_k, max_m, w)
+        assert blocks(max_k, max_m, 2**31 - 1) == whole
+    for w in widths:  # what the kernel computes with
+        assert 0 <= lib._ZN2tt12align_windowEi(w) <= binding.TT_MAX_K + binding.TT_MAX_M
