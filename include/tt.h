@@ -159,7 +159,10 @@ typedef struct {
   /* Histories of the repetition penalty (read only when that family's penalty
      is on): request b's earlier tokens as logits columns,
      hist_cols[hist_off[b] .. hist_off[b+1]), at most TT_MAX_HISTORY per request
-     (TT_REQ_TOO_LONG beyond); NULL hist_off = empty histories. */
+     (TT_REQ_TOO_LONG beyond); NULL hist_off = empty histories. Offsets must not
+     fall: a request with a bad range, or whose range and tokens would take the
+     place that offsets before a fall gave an earlier request, is reported as
+     TT_REQ_BAD_OFFSETS; the others are not affected. */
   const int32_t* hist_off_d;  /* [B+1] draft family (draft logits columns) */
   const int32_t* hist_cols_d; /* [n_hist_d] */
   const int32_t* hist_off_t;  /* [B+1] target family (target logits columns) */

@@ -37,6 +37,7 @@ struct PenSmem {
   int32_t bad;
 };
 
+// [lo, hi) = off[b] .. off[b + 1], empty when they are no range of [0, n).
 __device__ __forceinline__ bool csr_range(const int32_t* off, int b, int n, int& lo, int& hi) {
   lo = hi = 0;
   if (!off) return true;
@@ -50,6 +51,20 @@ __device__ __forceinline__ bool csr_range(const int32_t* off, int b, int n, int&
 // Barrier of one family's threads.
 __device__ __forceinline__ void family_sync(int fam) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + fam), "n"(kPT) : "memory");
+}
+
+// The same, and whether any of them passed true.
+__device__ __forceinline__ bool family_or(int fam, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.s32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.pred q, %2, %3, p;\n\t"
+      "selp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(int(p)), "r"(1 + fam), "n"(kPT)
+      : "memory");
+  return r != 0;
 }
 
 __global__ void __launch_bounds__(2 * kPT) pen_prep_kernel(PenArgs a) {
@@ -67,19 +82,26 @@ __global__ void __launch_bounds__(2 * kPT) pen_prep_kernel(PenArgs a) {
     const int nlist = tgt ? a.nlist_t : a.nlist_d;
     const int lg = 31 - __clz(tgt ? a.unit_t : a.unit_d);  // a unit's columns: a power of two
     const int nch = tgt ? a.nch_t : a.nch_d;
+    const int32_t* hoff = tgt ? a.hist_off_t : a.hist_off_d;
+    const int32_t* soff = tgt ? a.target_off : a.draft_off;
+    const int n_hist = tgt ? a.n_hist_t : a.n_hist_d, n_seq = tgt ? a.n_target : a.n_draft;
     int st = 0, h0, h1, s0, s1;
-    if (!csr_range(tgt ? a.hist_off_t : a.hist_off_d, b, tgt ? a.n_hist_t : a.n_hist_d, h0, h1)) {
-      st |= TT_REQ_BAD_OFFSETS;
-      h0 = h1 = 0;
-    }
-    if (!csr_range(tgt ? a.target_off : a.draft_off, b, tgt ? a.n_target : a.n_draft, s0, s1))
-      s0 = s1 = 0;  // (reported by the other kernels)
+    const bool h_ok = csr_range(hoff, b, n_hist, h0, h1), s_ok = csr_range(soff, b, n_seq, s0, s1);
+    if (!h_ok) st |= TT_REQ_BAD_OFFSETS;
+    // without both ranges the request has no segment to write entries to (a bad
+    // sequence range is reported by the other kernels)
+    if (!h_ok || !s_ok) h1 = h0, s1 = s0;
     if (h1 - h0 > TT_MAX_HISTORY) {
       st |= TT_REQ_TOO_LONG;
       h1 = h0;
     }
     if (s1 - s0 > TT_MAX_M) s1 = s0;  // (too long: reported by the other kernels)
-    const int nh = h1 - h0, n = nh + (s1 - s0);
+    int nh = h1 - h0, n = nh + (s1 - s0);
+    // Offsets that fall somewhere before this request (which one of them is bad)
+    // may put its segment over that of an earlier one.
+    bool fell = false;
+#pragma unroll 4
+    for (int x = tid; x < b; x += kPT) fell |= (hoff && hoff[x] > h0) || soff[x] > s0;
     const int32_t* hcols = (tgt ? a.hist_cols_t : a.hist_cols_d) + h0;
     const int32_t* scols = (tgt ? a.target_cols : a.draft_cols) + s0;
     int slots = 64;  // at least twice the entries where the table allows
@@ -87,7 +109,18 @@ __global__ void __launch_bounds__(2 * kPT) pen_prep_kernel(PenArgs a) {
     for (int i = tid; i < slots; i += kPT) sm.slot[i] = kEmpty;
     for (int u = tid; u < nlist; u += kPT) sm.count[u] = 0;
     if (tid == 0) sm.bad = 0;
-    family_sync(fam);
+    if (family_or(fam, fell && n > 0)) {
+      bool over = false;
+      for (int x = tid; x < b; x += kPT) {
+        int x0, x1, y0, y1;
+        if (csr_range(hoff, x, n_hist, x0, x1) && csr_range(soff, x, n_seq, y0, y1))
+          over |= max(x0 + y0, h0 + s0) < min(x1 + y1, h1 + s1);
+      }
+      if (family_or(fam, over)) {  // the earlier one keeps it
+        st |= TT_REQ_BAD_OFFSETS;
+        nh = n = 0;
+      }
+    }
     // one slot per column, holding the smallest first position (history: -1)
     constexpr int kFly = 4;  // columns in flight per thread
     for (int i0 = tid; i0 < n; i0 += kFly * kPT) {
@@ -124,7 +157,7 @@ __global__ void __launch_bounds__(2 * kPT) pen_prep_kernel(PenArgs a) {
     }
     family_sync(fam);
     // where each unit's entries start
-    const int base = h0 + s0;  // the request's segment (capacity n)
+    const int base = h0 + s0;  // the request's segment (capacity n; no other request's)
     int32_t* start = (tgt ? a.pstart_t : a.pstart_d) + int64_t(b) * (nch + 1);
     constexpr int kPer = kMaxChunksPerRow / kPT;
     int cnt[kPer], sum = 0;

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2510_15545_gb300 as tt
 from paper_2510_15545_gb300 import workload as W
 from _parity import compare, oracle_step, to_np
@@ -78,3 +79,48 @@ def test_sets_at_edges(V, dt_d, dt_t, families):
     g = to_np(tt.tt_step(inp["batch"], inp["vd"], inp["vt"], _padded(wl.draft_logits),
                          _padded(wl.target_logits), inp["params"]))
     compare(wl, g, oracle_step(wl, **f))
+
+
+def _with_offsets(wl, off):
+    """The workload with every family's history offsets replaced."""
+    return dataclasses.replace(wl, hist_off_t=np.array(off, np.int32),
+                               hist_off_d=np.array(off, np.int32))
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("bad,refused,off", [
+    # which request's range is bad, which others are refused, the offset after it
+    (1, (), [0, 60, 56, 180, 240, 300, 360]),     # request 2 reaches back, up to request 0's place
+    (1, (2,), [0, 60, 50, 180, 240, 300, 360]),   # ... and would take part of its place
+    (3, (4,), [0, 60, 120, 180, 0, 300, 360]),    # ... of three requests' places
+    (0, (), [-1, 60, 120, 180, 240, 300, 360]),
+    (5, (), [0, 60, 120, 180, 240, 300, 299]),
+])
+def test_a_bad_history_range_leaves_the_other_requests_alone(dt, bad, refused, off):
+    """A request without a usable history range writes no entries (it wrote its
+    tokens' entries at a place that belongs to an earlier request)."""
+    B, G, V = 6, 4, 9001
+    wl = W.homogeneous_workload(B, G, V, seed=3, logit_scale=2.5)
+    wl = dataclasses.replace(wl, draft_logits=wl.draft_logits.to(dt),
+                             target_logits=wl.target_logits.to(dt))
+    rng = np.random.default_rng(1)
+    # each request's history holds the leading columns of its rows
+    for fam, logits in (("d", wl.draft_logits), ("t", wl.target_logits)):
+        lead = torch.topk(logits.float().reshape(B, -1, V), 6, dim=2).indices.reshape(B, -1)
+        cols = np.concatenate([rng.permutation(x.numpy())[:20] for x in lead for _ in range(3)])
+        wl = dataclasses.replace(wl, **{"hist_cols_" + fam: cols.astype(np.int32)})
+    wl = _with_offsets(wl, off)
+    inp = tt.device_inputs(wl, "cuda")
+    inp["batch"].n_hist_d = inp["batch"].n_hist_t = 360
+    for k, v in PEN.items():
+        setattr(inp["params"], k, v)
+    g = to_np(tt.tt_step(inp["batch"], inp["vd"], inp["vt"], _padded(wl.draft_logits),
+                         _padded(wl.target_logits), inp["params"]))
+    for b in range(B):
+        if b == bad or b in refused or off[b] < 0 or off[b + 1] < off[b]:
+            assert g["status"][b] == oracle.ST_BAD_OFFSETS, b
+        else:  # as the request alone
+            sw = wl.subset([b])
+            o = oracle_step(sw, request_base=b, **PEN)
+            compare(sw, dict(g, _target_off=wl.target_off, _draft_off=wl.draft_off), o,
+                    req_index=[b])
