@@ -321,8 +321,12 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
     if (th2 >= kPairFloor && th2 < INFINITY) {
       // The terms are fp32 values (2^f from the SFU, the exponent split exactly),
       // so their prefix sums are taken in fp32 pairs; the hit is the first column
-      // whose running mass passes theta.
+      // with mass whose running mass passes theta. (A thread's `run` is added up
+      // in another order than the last sum of the thread before it: without the
+      // test of the column's own mass, one without any could be the first past
+      // theta by the last bit.)
       F2 mine = {0.f, 0.f}, next[kPer];
+      uint32_t mass = 0;  // the thread's columns that have any
 #pragma unroll
       for (int k = 0; k < kPer; ++k) {
         const int x = c0 + k;
@@ -335,7 +339,10 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
         }
         mine = f2_add(mine, w);
         next[k] = mine;
-        if (w.hi > 0.f) last = x;
+        if (w.hi > 0.f) {
+          last = x;
+          mass |= 1u << k;
+        }
       }
       F2 incl = mine;
 #pragma unroll
@@ -354,7 +361,7 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
       int hit = 0x7fffffff;
 #pragma unroll
       for (int k = kPer - 1; k >= 0; --k)
-        if (f2_lt(thp, f2_add(run, next[k]))) hit = c0 + k;
+        if ((mass >> k & 1u) && f2_lt(thp, f2_add(run, next[k]))) hit = c0 + k;
       hit = __reduce_min_sync(0xffffffffu, hit);
       if (lane == 0 && hit != 0x7fffffff) atomicMin(&s_hit, hit);
     } else {

@@ -61,3 +61,46 @@ def test_shards_of_both_types(B, G, widths, dtypes):
     o = oracle.verify(wl.target_off, wl.target_cols, q, whole, seed=prm.seed)
     g, o = dict(g, q_hat=q), dict(o, q_hat=q)
     compare(wl, g, o, check_align=False)
+
+
+# Seeds, and columns with -log2 of their masses (all others have none), of a
+# bonus row whose uniform falls between two roundings of one running mass: the
+# pair sum that a thread ends on is at or below it, the sum from which one of the
+# next threads starts, added up in another order, is above it by its last bit,
+# and that thread's first columns have no mass.
+BETWEEN = [
+    (99, {
+        18: 19, 28: 42, 32: 1, 51: 49, 55: 15, 57: 38, 320: 18, 427: 17, 447: 13, 505: 11,
+        513: 48, 550: 51, 561: 23, 601: 44, 645: 37, 683: 53, 713: 41, 718: 9, 761: 21, 796: 3,
+        880: 22, 914: 52, 920: 5, 1025: 12, 1067: 54, 1079: 50, 1089: 53, 1098: 54, 1140: 29,
+        1154: 32, 1161: 53, 1206: 47, 1620: 0}),
+    (220, {
+        42: 47, 149: 36, 165: 33, 259: 8, 267: 15, 343: 46, 502: 32, 560: 16, 569: 35, 600: 34,
+        695: 5, 752: 20, 765: 53, 769: 10, 804: 52, 817: 39, 824: 29, 841: 11, 853: 1, 1002: 28,
+        1126: 7, 1215: 23, 1282: 52, 1314: 40, 1330: 43, 1351: 21, 1364: 52, 1947: 0}),
+    (252, {
+        13: 16, 140: 17, 185: 40, 198: 31, 256: 8, 491: 34, 507: 47, 677: 9, 706: 53, 718: 36,
+        740: 37, 807: 12, 818: 43, 825: 3, 873: 13, 920: 23, 938: 30, 1022: 1, 1061: 33,
+        1094: 29, 1130: 5, 1190: 53, 2009: 0}),
+]
+
+
+@pytest.mark.parametrize("seed,masses", BETWEEN)
+def test_a_column_without_mass_is_never_drawn(seed, masses):
+    V = 2048
+    wl = W.homogeneous_workload(1, 1, V, seed=1)
+    z = torch.full((2, V), -float("inf"))
+    z[0] = 0.0
+    for c, e in masses.items():
+        z[1, c] = -float(e)
+    wl = dataclasses.replace(wl, target_logits=z)
+    inp = tt.device_inputs(wl, "cuda")
+    prm = inp["params"]
+    prm.seed, prm.temp_target = seed, float(np.log2(np.e))  # masses are 2^z exactly
+    q = torch.zeros(1, device="cuda")                       # the token is accepted
+    g = to_np(tt.tt_verify_sharded(inp["batch"], q, [z.to("cuda")], prm, summaries=True))
+    assert g["status"][0] == 0 and g["accepted"][0] == 1
+    # the row's total, against which the uniform is taken: the masses of 2^-23 and more
+    total = np.float32(sum(2.0 ** -e for e in masses.values() if e <= 23))
+    assert g["summaries"][0, 1, 0] == 0.0 and g["summaries"][0, 1, 1] == total
+    assert int(g["next_token"][0]) in masses
