@@ -204,6 +204,8 @@ __device__ __forceinline__ uint32_t apply_penalty(char* stage, const Desc& d, co
   };
   if (p.e.col >= 0) apply(p.e);
   for (int i = p.lo + 32 + lane; i < p.hi; i += 32) apply(S.pen[i]);
+  // the stage's next bulk copy comes after these writes, in the async proxy's view too
+  if (p.lo < p.hi) fence_proxy_async();
   tail = __reduce_or_sync(0xffffffffu, tail);
   __syncwarp();
   return tail;

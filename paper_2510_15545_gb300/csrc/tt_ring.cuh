@@ -50,6 +50,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   }
   return false;
 }
+// Orders this thread's shared-memory writes before bulk copies into the same
+// place that are issued after its next arrival: an mbarrier alone orders a copy
+// behind earlier reads, but not behind ordinary writes.
+__device__ __forceinline__ void fence_proxy_async() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 // Bulk copy of a piece of a streamed row. Rows are read once each: their lines
 // leave L2 first, and what is read again (partials, lists, tables, offsets)
 // stays: 64 requests (500 MB) 86.9 -> 84.5 us, filtered and sharded ones 3 % less,
