@@ -55,6 +55,21 @@ def test_widths_at_edges(V, dtype):
     _check(W.homogeneous_workload(4, 3, V, seed=V, dtype=dtype, logit_scale=2.5))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("sigma", [0.0, 0.3, 1.0, 2.0])
+def test_flat_rows_raise_their_bar(sigma, dtype):
+    """Every unit holds more candidates than a warp has room for, by some or by
+    all of its columns (equal logits: no bar leaves room), and a ragged unit."""
+    wl = W.homogeneous_workload(5, 3, 30005, seed=int(10 * sigma), logit_scale=max(sigma, 0.1))
+    if sigma == 0.0:
+        wl = dataclasses.replace(wl, draft_logits=torch.zeros_like(wl.draft_logits),
+                                 target_logits=torch.full_like(wl.target_logits, 2.0))
+    wl = dataclasses.replace(wl, draft_logits=wl.draft_logits.to(dtype),
+                             target_logits=wl.target_logits.to(dtype))
+    for p in (0.3, 0.95):
+        _check(wl, dict(LLAMA, top_p_draft=p, top_p_target=p))
+
+
 def test_families_of_different_types():
     wl = W.homogeneous_workload(6, 4, 20011, seed=3, logit_scale=2.5)
     _check(dataclasses.replace(wl, draft_logits=wl.draft_logits.to(torch.bfloat16)))
