@@ -155,7 +155,7 @@ cudaError_t launch_pen_sets(const tt_batch* batch, const RowSet& d, const RowSet
 }
 
 // A nucleus family's row set (see RowSet::nucleus).
-void attach_nucleus(RowSet& r, bool on) { r.nucleus = nucleus_rows(on, r.V); }
+void attach_nucleus(RowSet& r, bool on) { r.nucleus = nucleus_rows(on, r.V, r.unit_cols); }
 
 // Streams the rows of r: wide nucleus families by the nucleus row kernel, the
 // others by the row pass.

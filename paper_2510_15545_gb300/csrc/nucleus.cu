@@ -65,7 +65,7 @@ constexpr int kRetryCands = 3200;      // candidates a second pass may take (of 
 constexpr float kMinBar = 8.f;         // lowest bar of a second pass
 // Rows of at most kWarpRowMax columns: one warp per row (nucleus_warp_kernel),
 // candidates within kWCandDelta log2 units of the maximum, at most kWCap.
-constexpr int kWarpRowMax = kNucNarrow;
+constexpr int kWarpRowMax = 8192;
 constexpr float kWCandDelta = 12.f;
 constexpr int kWCap = 512;
 constexpr int kWBuckets = int(kWCandDelta) * 32 + 32;
@@ -680,10 +680,15 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
   }
 }
 
-// One CTA per nucleus row: the rows that the nucleus row kernel or
-// nucleus_warp_kernel left (head n = -1), found in tiles of at most 256 rows,
-// and every row of a family wider than either takes. Tiles of draft rows, then of target
-// rows, grid-stride.
+// Rows of which an earlier kernel (nucleus_warp_kernel or the nucleus row
+// kernel) has settled most.
+__device__ __forceinline__ bool settled_before(const RowSet& S) {
+  return S.V <= kWarpRowMax || S.nucleus == kNucWideRows;
+}
+
+// One CTA per nucleus row: the rows that an earlier kernel left (head n = -1),
+// found in tiles of at most 256 rows, and every row of the other families. Tiles
+// of draft rows, then of target rows, grid-stride.
 __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   extern __shared__ __align__(16) char nsm_raw[];
   NucSmem& sm = *reinterpret_cast<NucSmem*>(nsm_raw);
@@ -692,7 +697,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   // rows per tile: one when every row is to be done, else a share of the rows
   auto tile_rows = [&](const RowSet& S, int64_t rows) {
     const int64_t share = (rows + gridDim.x - 1) / gridDim.x;
-    return S.V <= kNucWideMax ? int(max(int64_t(1), min(int64_t(kNT), share))) : 1;
+    return settled_before(S) ? int(max(int64_t(1), min(int64_t(kNT), share))) : 1;
   };
   const int tsz_d = tile_rows(a.d, rows_d), tsz_t = tile_rows(a.t, rows_t);
   const int64_t nt_d = (rows_d + tsz_d - 1) / tsz_d, nt_t = (rows_t + tsz_t - 1) / tsz_t;
@@ -703,7 +708,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   const int tsz = tgt ? tsz_t : tsz_d;
   const int64_t r0 = (tgt ? tile - nt_d : tile) * tsz;
   int n_todo = 1;
-  const bool some = (tgt ? a.t.V : a.d.V) <= kNucWideMax;
+  const bool some = settled_before(tgt ? a.t : a.d);
   if (some) {  // the rows an earlier kernel could not settle
     __syncthreads();
     if (tid == 0) sm.n_todo = 0;
@@ -711,7 +716,8 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
     const int64_t rr = r0 + tid;
     const RowSet& SF = tgt ? a.t : a.d;
     const KeptHead* hf = tgt ? a.head_t : a.head_d;
-    if (tid < tsz && rr < (tgt ? rows_t : rows_d) && (tgt || !SF.need || SF.need[rr] != 0) && hf[rr].n == -1)
+    if (tid < tsz && rr < (tgt ? rows_t : rows_d) && (tgt || !SF.need || SF.need[rr] != 0) &&
+        hf[rr].n == -1)
       sm.todo[atomicAdd(&sm.n_todo, 1)] = tid;
     __syncthreads();
     n_todo = sm.n_todo;

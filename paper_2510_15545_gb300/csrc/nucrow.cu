@@ -1,5 +1,5 @@
 // nucrow.cu -- nucleus rows (top-p without top-k, App. F) of more than
-// kNucNarrow columns: every row streamed from HBM once and its kept set
+// kNucRowUnits units of 8 KB: every row streamed from HBM once and its kept set
 // found from what the CTA holds of it.
 //
 // One CTA per SM, three roles:

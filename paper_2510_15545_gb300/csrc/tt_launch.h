@@ -42,13 +42,23 @@ struct AlignArgs {
 
 constexpr int kNucNarrowRows = 1;  // RowSet::nucleus
 constexpr int kNucWideRows = 2;
-// How a nucleus family's rows of V columns are settled: rows of more than
-// kNucNarrow columns (and at most kNucWideMax) by the nucleus row kernel.
-constexpr int kNucNarrow = 8192;
+// How a nucleus family's rows of V columns (unit_cols to an 8 KB unit) are
+// settled: rows of more than kNucRowUnits units, and at most kNucWideMax
+// columns, by the nucleus row kernel. It hands each unit to another of its
+// warps, so in rows of few units most warps and most of its room for candidates
+// stay unused. Against the row pass and the kernels after it, on Zipf logits
+// (both families of one width):
+//                        64 requests, top-p 0.95   512 requests, top-p 0.9
+//   bf16 10,000 (2.4 units)    115 us to 89             490 us to 441
+//   bf16 16,323 (4.0)          102 us to 97             447 us to 509
+//   bf16 20,419 (5.0)           98 us to 103            430 us to 580
+//   fp32  9,155 (4.5)           95 us to 96             409 us to 500
+//   fp32 16,323 (8.0)           92 us to 105            396 us to 569
+constexpr int kNucRowUnits = 4;
 constexpr int kNucWideMax = 480 * 2048;
-inline int nucleus_rows(bool nucleus, int V) {
+inline int nucleus_rows(bool nucleus, int V, int unit_cols) {
   if (!nucleus) return 0;
-  return V > kNucNarrow && V <= kNucWideMax ? kNucWideRows : kNucNarrowRows;
+  return V > kNucRowUnits * unit_cols && V <= kNucWideMax ? kNucWideRows : kNucNarrowRows;
 }
 
 // One family of logits rows seen by the row pass.
