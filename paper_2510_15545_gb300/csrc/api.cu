@@ -192,6 +192,19 @@ cudaError_t launch_rows(const RowPassArgs& r, const tt_params* prm, const Worksp
   return launch_nucleus_rows(n, dt_d, dt_t, s, sm_count_current(), pdl);
 }
 
+// Whether the streamed rows stay in L2 for the decision (RowPassArgs::keep): the
+// full-q residual reads a target and a draft row of each request again, unless
+// both are filtered (their kept sets are lists), and finds them there while
+// everything streamed fits beside the rest: three quarters of 129 MB. Full-q
+// steps of 24 requests (17 fp32 rows of 50,257 columns each, 82 MB in all) take
+// 182 us with rows that leave first and 133 us with rows that stay, of 32 (109 MB)
+// 186 and 193, of 128 234 and 258.
+constexpr int64_t kKeepBytes = 96 << 20;
+int32_t keep_rows(const RowPassArgs& r, const tt_params* prm) {
+  return prm->full_q && r.t.top_k == 0 &&
+         r.rows_t * r.t.stride_bytes + r.rows_d * r.d.stride_bytes <= kKeepBytes;
+}
+
 // A family's row set sees its penalty arrays.
 void attach_pen(RowSet& r, bool on, float theta, PenEntry* pen, const int32_t* pbase,
                 const int32_t* pcnt, const int32_t* pstart) {
@@ -620,6 +633,7 @@ tt_status tt_verify(const tt_batch* batch, const float* q_hat, const tt_logits* 
   r.epoch = next_epoch();
   r.work = full_q ? ws.work : nullptr;  // zeroed by the prep kernel
   r.pre_eighths = 4;
+  r.keep = keep_rows(r, prm);
   // the first kernel of the chain starts only after the caller's work is
   // complete: it reads the logits before its grid-dependency wait
   if ((e = launch_rows(r, prm, ws, full_q ? draft->dtype : target->dtype, target->dtype, s,
@@ -748,6 +762,7 @@ tt_status tt_step(const tt_batch* batch, const tt_vocab* vd, const tt_vocab* vt,
   r.work = ws.work;       // zeroed by the alignment kernel
   r.pre_eighths = 4;
   r.excl_late = ws.excl;  // written by the alignment kernel
+  r.keep = keep_rows(r, prm);
   // programmatic dependent launch: target rows stream while the alignment runs
   // (unless stage events sit between the kernels)
   const bool pdl = prm->events == nullptr;

@@ -50,6 +50,9 @@ struct Desc {
 // type in one grid, so that one ring fill and one tail serve them all. Four
 // shards of 64 requests (436 MB) took four passes of 23 us in turn, 68 us now.
 constexpr int kShards = 3;
+// The plain variant with streamed rows that stay in L2 (RowPassArgs::keep). A
+// choice at each copy of the one kernel took 1.2 % of the 1024-request step.
+constexpr int kKeep = 4;
 
 // Stage s is always refilled for the same consumer warp (s mod kConsumerWarps),
 // so a warp never waits on a stage more than one phase ahead of it: an
@@ -762,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         if (penalties) mbar_arrive(&posted[s]);
         if (copy_ok && bytes > 0) {
           mbar_arrive_expect_tx(&full[s], bytes);
-          bulk_copy_g2s(stages + size_t(s) * R::kStageBytes, src, bytes, &full[s]);
+          bulk_copy_g2s<SEL != kKeep>(stages + size_t(s) * R::kStageBytes, src, bytes, &full[s]);
         } else {
           mbar_arrive(&full[s]);
         }
@@ -1043,18 +1046,21 @@ cudaError_t launch_rowpass_t(const PassArgs<SEL>& a, cudaStream_t stream, int sm
 template <int DTD, int DTT>
 cudaError_t preload_pair() {
   cudaError_t e = preload_t<DTD, DTT, 0>();
+  if (e == cudaSuccess) e = preload_t<DTD, DTT, kKeep>();
   if (e == cudaSuccess) e = preload_t<DTD, DTT, 1>();
   return e != cudaSuccess ? e : preload_t<DTD, DTT, 2>();
 }
 
-// Variants: 0 partials only; 1 top-k lists for filtered families; 2 lists with
-// the repetition penalty and the nucleus rows' partials (kept apart
-// so that plain filtered rows run the smaller consumer loop).
+// Variants: 0 partials only (kKeep: of rows that stay in L2); 1 top-k lists for
+// filtered families; 2 lists with the repetition penalty and the nucleus rows'
+// partials (kept apart so that plain filtered rows run the smaller consumer
+// loop).
 template <int DTD, int DTT>
 cudaError_t launch_pair(const RowPassArgs& a, cudaStream_t stream, int sm_count, bool pdl) {
   if (a.d.pen || a.t.pen || a.d.nucleus || a.t.nucleus)
     return launch_rowpass_t<DTD, DTT, 2>(a, stream, sm_count, pdl);
   if (a.d.top_k > 0 || a.t.top_k > 0) return launch_rowpass_t<DTD, DTT, 1>(a, stream, sm_count, pdl);
+  if (a.keep) return launch_rowpass_t<DTD, DTT, kKeep>(a, stream, sm_count, pdl);
   return launch_rowpass_t<DTD, DTT, 0>(a, stream, sm_count, pdl);
 }
 

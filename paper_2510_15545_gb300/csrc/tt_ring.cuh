@@ -56,23 +56,31 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-// Bulk copy of a piece of a streamed row. Rows are read once each: their lines
-// leave L2 first, and what is read again (partials, lists, tables, offsets)
-// stays: 64 requests (500 MB) 86.9 -> 84.5 us, filtered and sharded ones 3 % less,
-// batches of GBs the same. (The policy is formed at each copy: held in
+// Bulk copy of a piece of a streamed row. ONCE: the row is read once, and its
+// lines leave L2 first, so that what is read again (partials, lists, tables,
+// offsets) stays: 64 requests (500 MB) 86.9 -> 84.5 us, filtered and sharded ones
+// 3 % less, batches of GBs the same. (The policy is formed at each copy: held in
 // registers, it took the row pass past what lets a decision CTA sit beside it,
 // 96 us.)
+template <bool ONCE = true>
 __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes,
                                               uint64_t* bar) {
-  asm volatile(
-      "{\n"
-      ".reg .b64 once;\n"
-      "createpolicy.fractional.L2::evict_first.b64 once, 1.0;\n"
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1], %2, [%3], once;\n"
-      "}" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
+  if constexpr (ONCE) {
+    asm volatile(
+        "{\n"
+        ".reg .b64 once;\n"
+        "createpolicy.fractional.L2::evict_first.b64 once, 1.0;\n"
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1], %2, [%3], once;\n"
+        "}" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+  } else {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+        ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+  }
 }
 __device__ __forceinline__ void grid_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -197,6 +197,21 @@ def test_verify_full_q_matches_oracle():
     print(c)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("mb", [90, 102])
+def test_full_q_steps_around_the_l2_line(mb, dtype):
+    """Rows of up to 96 MB stay in L2 for the full-q residual, more leave it: a
+    variant of the row pass for either."""
+    k, V = 3, 60000
+    B = round(mb * 2**20 / ((2 * k + 1) * V * torch.empty(0, dtype=dtype).element_size()))
+    wl = W.homogeneous_workload(B, k, V, seed=mb, dtype=dtype, device="cuda")
+    g = gpu_step(wl, full_q=True)
+    for b in (0, B // 2, B - 1):
+        sw = wl.subset([b])
+        o = oracle_step(sw, full_q=True, request_base=b)
+        compare(sw, dict(g, _target_off=wl.target_off, _draft_off=wl.draft_off), o, req_index=[b])
+
+
 def test_verify_status_codes():
     V = 64
     t_off = np.array([0, 2, 2, 3, 5], np.int32)
