@@ -189,8 +189,49 @@ def crowded_rows(wl, seed=21):
 
 
 def test_rows_that_overflow_the_first_candidate_bar():
-    """The nucleus kernel's second candidate pass (a lower whole bar estimated
-    from the held candidates) settles these rows; compared with the oracle."""
+    """The row kernel's full regions raise their bars and settle these rows;
+    compared with the oracle."""
     wl = crowded_rows(_wl("b64_g8_v152k", 6, seed=13))
     f = dict(temp_target=0.6, top_p_target=0.5)
+    compare(wl, gpu_step(wl, **f), oracle_step(wl, **f))
+
+
+LEFT_TOP_P = 0.5
+
+
+def left_rows(wl, kind, dtype, seed=22):
+    """Target logits whose rows the nucleus row kernel leaves at T = 0.6 and
+    top-p 0.5 (log2 units below a column at the maximum; the rest far below):
+    "bucket": 200 columns of one 1/32-unit bucket, the cut among them;
+    "unit": 2048 columns of one 8 KB unit 1 to 9 units below, the cut past more of
+    them than a region holds, and 5000 columns at 12.5 to 13.5, so that a pass over
+    14 units overflows as well;
+    "crowd": 30,000 columns 1 to 5 units below."""
+    rng = np.random.default_rng(seed)
+    R, V = wl.target_logits.shape
+    scale = 1.4426950408889634 / 0.6
+    z = np.full((R, V), -40.0, np.float32)
+    for r in range(R):
+        if kind == "bucket":
+            cols = rng.permutation(V)[:201]
+            z[r, cols[1:]] = -(4.0 + rng.uniform(0.008, 0.012, 200)) / scale
+        elif kind == "unit":
+            n = 2048 if dtype == torch.float32 else 4096
+            cols = np.concatenate([[17], 3 * n + rng.permutation(n)[:2048]])
+            z[r, cols[1:]] = -rng.uniform(1.0, 9.0, 2048) / scale
+            far = rng.permutation(np.arange(5 * n, V))[:5000]
+            z[r, far] = -rng.uniform(12.5, 13.5, 5000) / scale
+        else:
+            cols = rng.permutation(V)[:30001]
+            z[r, cols[1:]] = -rng.uniform(1.0, 5.0, 30000) / scale
+        z[r, cols[0]] = 0.0
+    return dataclasses.replace(wl, target_logits=torch.as_tensor(z).to(dtype))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("kind", ["bucket", "unit", "crowd"])
+def test_rows_that_the_row_kernel_leaves(kind, dtype):
+    """Settled by the CTA kernel's first pass, its second and its levels in turn."""
+    wl = left_rows(_wl("b64_g8_v152k", 3, seed=13), kind, dtype)
+    f = dict(temp_target=0.6, top_p_target=LEFT_TOP_P)
     compare(wl, gpu_step(wl, **f), oracle_step(wl, **f))

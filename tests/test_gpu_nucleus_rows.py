@@ -16,7 +16,7 @@ import torch
 
 import paper_2510_15545_gb300 as tt
 from paper_2510_15545_gb300 import workload as W
-from _parity import compare, oracle_step, to_np
+from _parity import compare, gpu_step, oracle_step, to_np
 
 pytestmark = pytest.mark.gpu
 LLAMA = dict(temp_draft=0.6, temp_target=0.6, top_p_draft=0.9, top_p_target=0.9)
@@ -55,6 +55,29 @@ def _check(wl, f=LLAMA):
                                83967, 122887])
 def test_widths_at_edges(V, dtype):
     _check(W.homogeneous_workload(4, 3, V, seed=V, dtype=dtype, logit_scale=2.5))
+
+
+@pytest.mark.parametrize("V", [983040, 983041])
+def test_widths_around_the_widest(V):
+    """The widest rows of the row kernel, and the first that go past it."""
+    _check(W.homogeneous_workload(1, 2, V, seed=3, logit_scale=2.5))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [8199, 20011, 40961, 81919])
+def test_many_rows_per_cta(V, dtype):
+    """Nine rows and more on each CTA: the row buffers and the queue are used
+    again and again, short last rounds move from warp to warp, and rows are
+    expected to reach the maxima of those before them."""
+    wl = W.homogeneous_workload(200, 3, V, seed=V, dtype=dtype, logit_scale=2.5, device="cuda")
+    assert 7 * wl.B >= 9 * torch.cuda.get_device_properties(0).multi_processor_count
+    g = gpu_step(dataclasses.replace(wl, draft_logits=_padded(wl.draft_logits),
+                                     target_logits=_padded(wl.target_logits)), **LLAMA)
+    assert np.all(g["status"] == 0)
+    g["_target_off"], g["_draft_off"] = wl.target_off, wl.draft_off
+    for b in np.random.default_rng(V).choice(wl.B, size=12, replace=False):
+        sw = wl.subset([b])
+        compare(sw, dict(g), oracle_step(sw, request_base=int(b), **LLAMA), req_index=[b])
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
