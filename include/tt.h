@@ -354,9 +354,10 @@ tt_status tt_dpos_hist(const tt_batch* batch, const int32_t* path, const int32_t
  * residual row's mass per shard picks the shard that holds the drawn point,
  * and only that shard's slice is read again to find the column.
  * tt_verify_sharded runs that protocol with the S shards as S logits arrays on
- * one device: each shard's slice is reduced by its own row pass, and the
- * gathered summaries are a device buffer in the layout an all-gather would
- * produce ([S][n_target + B] records of 16 bytes). Results equal tt_verify's
+ * one device: one row pass per logits type reduces every shard's slice, each to
+ * its own partials (what its rank would do), and the gathered summaries are a
+ * device buffer in the layout an all-gather would produce ([S][n_target + B]
+ * records of 16 bytes). Results equal tt_verify's
  * on the concatenated rows up to rounding (same uniforms, same column order).
  * One-hot transfer only, no sampling filters (TT_ERR_UNSUPPORTED otherwise).
  */

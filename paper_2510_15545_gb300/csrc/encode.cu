@@ -291,7 +291,7 @@ struct FinArgs {
 };
 
 constexpr int kFinThreads = 256;
-constexpr int kFinCtas = 152;  // one per SM
+constexpr int kFinCtas = 152;  // one per SM of a GB300 (any number gives the same result)
 
 // Inclusive block scan of one int64 per thread; returns the block total in *total.
 __device__ int64_t block_scan(int64_t v, int64_t* s_warp, int64_t* total) {

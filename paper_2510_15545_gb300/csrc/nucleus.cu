@@ -539,7 +539,8 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
-      T = f2_add(T, F2{__shfl_xor_sync(0xffffffffu, T.hi, o), __shfl_xor_sync(0xffffffffu, T.lo, o)});
+      T = f2_add(T, F2{__shfl_xor_sync(0xffffffffu, T.hi, o),
+                       __shfl_xor_sync(0xffffffffu, T.lo, o)});
     const double Td = double(T.hi) + double(T.lo);
     if (!(Td > 0.0) || !isfinite(Td)) {
       if (lane == 0) head->n = -1;
@@ -796,8 +797,8 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
 
     float tau = -INFINITY;
     int tau_col = 0x7fffffff;  // all kept: every column ranks before (tau, tau_col)
-    const bool settled = candidate_cut(double(T.hi) + double(T.lo), sm, row, dt, V, nvec, vec, nch, M,
-                                       scale, top_p, tau, tau_col);
+    const bool settled = candidate_cut(double(T.hi) + double(T.lo), sm, row, dt, V, nvec, vec,
+                                       nch, M, scale, top_p, tau, tau_col);
     if (!settled) {
     // ------------------------------------- the crossing bucket, level by level
     Path cross;

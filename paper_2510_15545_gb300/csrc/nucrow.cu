@@ -246,7 +246,8 @@ __device__ __forceinline__ void comp_add2(uint64_t& hs, uint64_t& ls, uint64_t x
 __device__ __forceinline__ float comp_reduce(float hs, float ls) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, hs, o), ol = __shfl_xor_sync(0xffffffffu, ls, o);
+    const float oh = __shfl_xor_sync(0xffffffffu, hs, o);
+    const float ol = __shfl_xor_sync(0xffffffffu, ls, o);
     ls = __fadd_rn(ls, ol);
     comp_add(hs, ls, oh);
   }

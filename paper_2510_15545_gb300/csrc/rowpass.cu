@@ -12,8 +12,9 @@
 // chunks into a ring of shared-memory stages with 1-D bulk copies
 // (cp.async.bulk, completion counted on an mbarrier per stage); each of the 8
 // consumer warps owns every 8th stage, reduces one whole chunk at a time from
-// shared memory (no block barrier) and frees the stage. Every wait is bounded in time; on timeout the kernel sets
-// an error word that the decision kernel turns into a per-request status.
+// shared memory (no block barrier) and frees the stage. Every wait is bounded in
+// time; on timeout the kernel sets an error word that the decision kernel turns
+// into a per-request status.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
@@ -381,7 +382,8 @@ __device__ __forceinline__ Partial nuc_chunk_partial(const char* stage, const De
     if (zt > -INFINITY) add(ex2_approx(fmaf(zt, scale, -m)));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, hs, o), ol = __shfl_xor_sync(0xffffffffu, ls, o);
+      const float oh = __shfl_xor_sync(0xffffffffu, hs, o);
+      const float ol = __shfl_xor_sync(0xffffffffu, ls, o);
       ls = __fadd_rn(ls, ol);
       add(oh);
     }
@@ -720,9 +722,8 @@ __global__ void __launch_bounds__(kThreads, 3)
           cps = R::kCpsT;
           if (SEL != kShards && row != cached_row) {
             cached_row = row;
-            cached_excl = a.excl                ? a.excl[row]
-                          : (late && a.excl_late) ? a.excl_late[row]
-                                                  : excl_lookup(a, &cursor, row);
+            cached_excl =
+                late && a.excl_late ? a.excl_late[row] : excl_lookup(a, &cursor, row);
           }
           const int ex = cached_excl - unit * cps * kChunk;
           d.excl = (cached_excl >= 0 && ex >= 0 && ex < cps * kChunk) ? ex : -1;
@@ -1059,7 +1060,8 @@ template <int DTD, int DTT>
 cudaError_t launch_pair(const RowPassArgs& a, cudaStream_t stream, int sm_count, bool pdl) {
   if (a.d.pen || a.t.pen || a.d.nucleus || a.t.nucleus)
     return launch_rowpass_t<DTD, DTT, 2>(a, stream, sm_count, pdl);
-  if (a.d.top_k > 0 || a.t.top_k > 0) return launch_rowpass_t<DTD, DTT, 1>(a, stream, sm_count, pdl);
+  if (a.d.top_k > 0 || a.t.top_k > 0)
+    return launch_rowpass_t<DTD, DTT, 1>(a, stream, sm_count, pdl);
   if (a.keep) return launch_rowpass_t<DTD, DTT, kKeep>(a, stream, sm_count, pdl);
   return launch_rowpass_t<DTD, DTT, 0>(a, stream, sm_count, pdl);
 }
@@ -1122,9 +1124,12 @@ cudaError_t launch_rowpass(const RowPassArgs& args, int dt_d, int dt_t, cudaStre
                            int sm_count, bool pdl) {
   RowPassArgs a = args;
   next_launch_stall(&a.stall_stage, &a.wait_ns);
-  if (dt_d == TT_F32 && dt_t == TT_F32) return launch_pair<TT_F32, TT_F32>(a, stream, sm_count, pdl);
-  if (dt_d == TT_F32 && dt_t == TT_BF16) return launch_pair<TT_F32, TT_BF16>(a, stream, sm_count, pdl);
-  if (dt_d == TT_BF16 && dt_t == TT_F32) return launch_pair<TT_BF16, TT_F32>(a, stream, sm_count, pdl);
+  if (dt_d == TT_F32 && dt_t == TT_F32)
+    return launch_pair<TT_F32, TT_F32>(a, stream, sm_count, pdl);
+  if (dt_d == TT_F32 && dt_t == TT_BF16)
+    return launch_pair<TT_F32, TT_BF16>(a, stream, sm_count, pdl);
+  if (dt_d == TT_BF16 && dt_t == TT_F32)
+    return launch_pair<TT_BF16, TT_F32>(a, stream, sm_count, pdl);
   return launch_pair<TT_BF16, TT_BF16>(a, stream, sm_count, pdl);
 }
 

@@ -4,15 +4,15 @@
 //
 // A row pass over the slices (one grid for all shards of a type; per shard it is
 // what one rank does) gives chunk partials with the scored token left out;
-// shard_summary_kernel
-// reduces them to one record per row (max, sum of 2^(s - max) as an fp64 pair
-// of floats, the owned scored token's scaled logit or NaN). The records of all
-// shards are the exchange (an all-gather across ranks; here a device buffer in
-// that layout). decide_sharded_kernel merges them (split-lse), runs the accept
-// test with the same Philox uniforms as the unsharded path, and samples the
-// residual (or the bonus row) by inverse CDF in column order at three levels:
-// the shard from the merged records, the chunk within that shard from its
-// partials, and the column from one re-read chunk of that shard's slice.
+// shard_summary_kernel reduces them to one record per row (max, sum of
+// 2^(s - max) as an fp64 pair of floats, the owned scored token's scaled logit or
+// NaN). The records of all shards are the exchange (an all-gather across ranks;
+// here a device buffer in that layout). decide_sharded_kernel merges them
+// (split-lse), runs the accept test with the same Philox uniforms as the
+// unsharded path, and samples the residual (or the bonus row) by inverse CDF in
+// column order at three levels: the shard from the merged records, the chunk
+// within that shard from its partials, and the column from one re-read chunk of
+// that shard's slice.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -95,8 +95,8 @@ __global__ void shard_summary_kernel(ShardArgs a) {
       float st = __int_as_float(0x7fffffff);
       if (x >= 0) {
         const char* row = d.data + r * d.stride_bytes;
-        const float z = d.dtype == TT_F32 ? load_logit<TT_F32>(row, x) : load_logit<TT_BF16>(row, x);
-        st = z * a.scale;
+        st = (d.dtype == TT_F32 ? load_logit<TT_F32>(row, x) : load_logit<TT_BF16>(row, x)) *
+             a.scale;
       }
       const float hi = float(Ssum);
       a.rec[w] = ShardRec{M, hi, float(Ssum - double(hi)), st};
@@ -313,9 +313,10 @@ __global__ void __launch_bounds__(kShThreads) decide_sharded_kernel(ShardArgs a)
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int x = c0 + k;
-      z[k] = x >= d.V ? -INFINITY
-                      : (d.dtype == TT_F32 ? load_logit<TT_F32>(rp, x) : load_logit<TT_BF16>(rp, x)) *
-                            a.scale;
+      z[k] = -INFINITY;
+      if (x < d.V)
+        z[k] = (d.dtype == TT_F32 ? load_logit<TT_F32>(rp, x) : load_logit<TT_BF16>(rp, x)) *
+               a.scale;
     }
     int last = -1;
     if (th2 >= kPairFloor && th2 < INFINITY) {

@@ -1,6 +1,7 @@
 // tt_f2.cuh -- compensated fp32 pairs (an unevaluated sum hi + lo, about
-// 2^-44 relative), 2^y with an exact exponent split, and the grid-dependency
-// wait, shared by the decision kernels (decide.cu, filter.cu).
+// 2^-44 relative), 2^y with an exact exponent split, the normaliser of a nucleus
+// row's kept set, and the grid-dependency wait: shared by the kernels of all
+// stages.
 #pragma once
 
 #include "tt_device.cuh"

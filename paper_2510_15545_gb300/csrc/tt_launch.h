@@ -93,16 +93,16 @@ struct RowSet {
 struct RowPassArgs {
   RowSet d, t;
   int64_t rows_d, rows_t;    // rows of each family to stream (0 = family absent)
-  const int32_t* excl;       // [target rows] column left out of the sum, or NULL: found
-                             // from target_off / target_cols
   int B, n_target, n_draft;
   const int32_t* target_off;
   const int32_t* target_cols;
   const int32_t* draft_off;  // to find a penalized draft row's request
   int32_t* err;              // err[0] = epoch of a failed call, err[1] = its TT_REQ_* bits
   int32_t epoch;             // identifies this call
-  const int32_t* excl_late;  // as excl, but written by the grid this one depends on: read
-                             // only after the grid-dependency wait (may be NULL)
+  const int32_t* excl_late;  // [target rows] column left out of the sum, written by the grid
+                             // this one depends on: read only after the grid-dependency
+                             // wait, before it (and when NULL) found from target_off /
+                             // target_cols
   // Work counter for the items past each CTA's fixed share, zeroed by the grid
   // this one depends on and read only after the grid-dependency wait; NULL:
   // every item belongs to a fixed share.
