@@ -125,7 +125,7 @@ struct NucSmem {
   int n_gc;
   int wn[kNW];  // candidates per warp region
   float ucnt[kUnitBins];  // estimated candidates per whole log2 unit of delta
-  int todo[kNT];  // rows of the current tile left to this kernel
+  int todo[kNT];  // of the rows looked at together, those to be done
   int n_todo;
   float tau_v;  // the last kept column, found by one warp
   int tau_c;
@@ -687,46 +687,39 @@ __device__ __forceinline__ bool settled_before(const RowSet& S) {
   return S.V <= kWarpRowMax || S.nucleus == kNucWideRows;
 }
 
-// One CTA per nucleus row: the rows that an earlier kernel left (head n = -1),
-// found in tiles of at most 256 rows, and every row of the other families. Tiles
-// of draft rows, then of target rows, grid-stride.
+// One CTA per nucleus row: the rows that an earlier kernel left (head n = -1) and
+// every row of the other families. CTA c takes rows c, c + G, ... of the draft
+// and then the target rows, 256 of them looked at together, so that rows left in
+// numbers spread over all CTAs. (In tiles of neighbouring rows, a tile per CTA
+// and family, a step of 1032 flat rows of 151,936 bf16 columns took 3048 us; 2349
+// now.)
 __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
   extern __shared__ __align__(16) char nsm_raw[];
   NucSmem& sm = *reinterpret_cast<NucSmem*>(nsm_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t rows_d = a.d.nucleus ? a.rows_d : 0, rows_t = a.t.nucleus ? a.rows_t : 0;
-  // rows per tile: one when every row is to be done, else a share of the rows
-  auto tile_rows = [&](const RowSet& S, int64_t rows) {
-    const int64_t share = (rows + gridDim.x - 1) / gridDim.x;
-    return settled_before(S) ? int(max(int64_t(1), min(int64_t(kNT), share))) : 1;
-  };
-  const int tsz_d = tile_rows(a.d, rows_d), tsz_t = tile_rows(a.t, rows_t);
-  const int64_t nt_d = (rows_d + tsz_d - 1) / tsz_d, nt_t = (rows_t + tsz_t - 1) / tsz_t;
   grid_dependency_wait();  // the partials (and the need flags) come from earlier kernels
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int64_t tile = blockIdx.x; tile < nt_d + nt_t; tile += gridDim.x) {
-  const bool tgt = tile >= nt_d;
-  const int tsz = tgt ? tsz_t : tsz_d;
-  const int64_t r0 = (tgt ? tile - nt_d : tile) * tsz;
-  int n_todo = 1;
-  const bool some = settled_before(tgt ? a.t : a.d);
-  if (some) {  // the rows an earlier kernel could not settle
-    __syncthreads();
-    if (tid == 0) sm.n_todo = 0;
-    __syncthreads();
-    const int64_t rr = r0 + tid;
-    const RowSet& SF = tgt ? a.t : a.d;
-    const KeptHead* hf = tgt ? a.head_t : a.head_d;
-    if (tid < tsz && rr < (tgt ? rows_t : rows_d) && (tgt || !SF.need || SF.need[rr] != 0) &&
-        hf[rr].n == -1)
-      sm.todo[atomicAdd(&sm.n_todo, 1)] = tid;
-    __syncthreads();
-    n_todo = sm.n_todo;
-  }
-  for (int k = 0; k < n_todo; ++k) {
-    const int64_t r = some ? r0 + sm.todo[k] : r0;
+  for (int64_t x0 = blockIdx.x; x0 < rows_d + rows_t; x0 += int64_t(kNT) * gridDim.x) {
+  __syncthreads();  // the list is reused
+  if (tid == 0) sm.n_todo = 0;
+  __syncthreads();
+  const int64_t mine = x0 + int64_t(tid) * gridDim.x;
+  if (mine < rows_d + rows_t) {
+    const bool tgt = mine >= rows_d;
+    const int64_t r = tgt ? mine - rows_d : mine;
     const RowSet& S = tgt ? a.t : a.d;
-    if (!tgt && S.need && S.need[r] == 0) continue;
+    if ((tgt || !S.need || S.need[r] != 0) &&
+        (!settled_before(S) || (tgt ? a.head_t : a.head_d)[r].n == -1))
+      sm.todo[atomicAdd(&sm.n_todo, 1)] = tid;
+  }
+  __syncthreads();
+  const int n_todo = sm.n_todo;
+  for (int k = 0; k < n_todo; ++k) {
+    const int64_t x = x0 + int64_t(sm.todo[k]) * gridDim.x;
+    const bool tgt = x >= rows_d;
+    const int64_t r = tgt ? x - rows_d : x;
+    const RowSet& S = tgt ? a.t : a.d;
     const int dt = tgt ? a.dt_t : a.dt_d;
     const float top_p = tgt ? a.top_p_t : a.top_p_d;
     KeptHead* head = (tgt ? a.head_t : a.head_d) + r;

@@ -235,3 +235,21 @@ def test_rows_that_the_row_kernel_leaves(kind, dtype):
     wl = left_rows(_wl("b64_g8_v152k", 3, seed=13), kind, dtype)
     f = dict(temp_target=0.6, top_p_target=LEFT_TOP_P)
     compare(wl, gpu_step(wl, **f), oracle_step(wl, **f))
+
+
+@pytest.mark.parametrize("V,B,k", [(64, 20000, 3), (9000, 300, 2)])
+def test_many_rows_left_to_the_cta_kernel(V, B, k):
+    """More rows left than CTAs (rows of tied logits: the cut's bucket holds too
+    many), of both families, every third row settled before; and more rows than
+    the CTAs look at in one go."""
+    wl = W.homogeneous_workload(B, k, V, seed=V, device="cuda", logit_scale=2.0)
+    for z in (wl.draft_logits, wl.target_logits):
+        z.copy_(torch.where(torch.arange(z.shape[0], device="cuda")[:, None] % 3 == 0, z,
+                            z.round().clamp_(-1, 1)))
+    g = gpu_step(wl, **LLAMA)
+    assert np.all(g["status"] == 0)
+    g["_target_off"], g["_draft_off"] = wl.target_off, wl.draft_off
+    for b in np.random.default_rng(V).choice(B, size=40, replace=False):
+        sw = sub_workload(wl, [b])
+        o = oracle_step(sw, request_base=int(b), **LLAMA)
+        compare(sw, dict(g), o, req_index=[b])
