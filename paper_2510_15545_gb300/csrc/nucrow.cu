@@ -446,44 +446,49 @@ __device__ __forceinline__ void stream_unit(const char* stage, const NrDesc& d, 
   // The candidates, appended to the warp's region: the flagged vectors are
   // listed, then their elements tested one per lane.
   for (float bar = kCandDelta;;) {
-    int n = st.n;
-    const bool tail = zt > zc;
-    const unsigned mt = __ballot_sync(0xffffffffu, tail);
-    if (tail && n + __popc(mt & ((1u << lane) - 1u)) < kRegion)
-      region[n + __popc(mt & ((1u << lane) - 1u))] = Cand{zt, d.col0 + d.n_smem + lane};
-    n += __popc(mt);
-    for (uint32_t f = flags; n <= kRegion && __any_sync(0xffffffffu, f != 0u);) {
-      if (lane == 0) list->n = 0;
-      __syncwarp();
-      int i = f ? atomicAdd(&list->n, __popc(f)) : kListed;
-      for (; f && i < kListed; f &= f - 1, ++i) list->v[i] = uint16_t((__ffs(f) - 1) * 32 + lane);
-      __syncwarp();
-      const int nv = min(list->n, kListed);
-      constexpr int kBatch = 4;  // elements in flight per lane
-      for (int k = 0; k < nv; k += kBatch * 32 / VEC) {
-        int x[kBatch];
-        float z[kBatch];
+    // (each flagged vector holds one at least: what cannot fit is not gathered)
+    int n = st.n + int(__reduce_add_sync(0xffffffffu, unsigned(__popc(flags))));
+    if (n <= kRegion) {
+      n = st.n;
+      const bool tail = zt > zc;
+      const unsigned mt = __ballot_sync(0xffffffffu, tail);
+      if (tail && n + __popc(mt & ((1u << lane) - 1u)) < kRegion)
+        region[n + __popc(mt & ((1u << lane) - 1u))] = Cand{zt, d.col0 + d.n_smem + lane};
+      n += __popc(mt);
+      for (uint32_t f = flags; n <= kRegion && __any_sync(0xffffffffu, f != 0u);) {
+        if (lane == 0) list->n = 0;
+        __syncwarp();
+        int i = f ? atomicAdd(&list->n, __popc(f)) : kListed;
+        for (; f && i < kListed; f &= f - 1, ++i)
+          list->v[i] = uint16_t((__ffs(f) - 1) * 32 + lane);
+        __syncwarp();
+        const int nv = min(list->n, kListed);
+        constexpr int kBatch = 4;  // elements in flight per lane
+        for (int k = 0; k < nv; k += kBatch * 32 / VEC) {
+          int x[kBatch];
+          float z[kBatch];
 #pragma unroll
-        for (int q = 0; q < kBatch; ++q) {
-          const int e = k + q * (32 / VEC) + lane / VEC;
-          x[q] = e < nv ? list->v[e] * VEC + lane % VEC : -1;
-        }
+          for (int q = 0; q < kBatch; ++q) {
+            const int e = k + q * (32 / VEC) + lane / VEC;
+            x[q] = e < nv ? list->v[e] * VEC + lane % VEC : -1;
+          }
 #pragma unroll
-        for (int q = 0; q < kBatch; ++q) {
-          const int y = max(x[q], 0);
-          z[q] = DT == TT_F32 ? reinterpret_cast<const float*>(stage)[y]
-                              : bf16_to_f32(reinterpret_cast<const uint16_t*>(stage)[y]);
-        }
+          for (int q = 0; q < kBatch; ++q) {
+            const int y = max(x[q], 0);
+            z[q] = DT == TT_F32 ? reinterpret_cast<const float*>(stage)[y]
+                                : bf16_to_f32(reinterpret_cast<const uint16_t*>(stage)[y]);
+          }
 #pragma unroll
-        for (int q = 0; q < kBatch; ++q) {
-          const bool take = x[q] >= 0 && z[q] > zc;
-          const unsigned m = __ballot_sync(0xffffffffu, take);
-          const int at = n + __popc(m & ((1u << lane) - 1u));
-          if (take && at < kRegion) region[at] = Cand{z[q], d.col0 + x[q]};
-          n += __popc(m);
+          for (int q = 0; q < kBatch; ++q) {
+            const bool take = x[q] >= 0 && z[q] > zc;
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            const int at = n + __popc(m & ((1u << lane) - 1u));
+            if (take && at < kRegion) region[at] = Cand{z[q], d.col0 + x[q]};
+            n += __popc(m);
+          }
         }
+        __syncwarp();
       }
-      __syncwarp();
     }
     if (n <= kRegion) {
       st.n = n;
