@@ -26,8 +26,8 @@
 // candidates while its share of the SM streamed nothing) moved every row twice:
 // 1133 + 1920 us for a step of 1024 requests (19,000 bf16 rows of 151,936 and
 // 201,088 columns, 7.0 GB; top-p 0.9), 78 + 131 us for 64 (fp32, 0.5 GB). This
-// one takes 1500 and 115 us. A unit costs about 1500 warp instructions, 1050 of
-// them for maxima and sums, at 61 % of the issue slots: it is bound by those
+// one takes 1436 and 109 us. A unit costs about 1500 warp instructions, 1050 of
+// them for maxima and sums, at 68 % of the issue slots: it is bound by those
 // and by the dependent chain of a unit's candidates (without candidates it
 // streams at 6.2 TB/s).
 #include <algorithm>
@@ -99,16 +99,36 @@ struct NrRow {  // one of the two rows in flight
   uint32_t best;  // key of the largest logit seen so far
 };
 
+// Sums of masses (whole numbers up to 2^40), each held as the sums of its lower 20
+// bits and of the others: kSW * kRegion terms do not overflow 32 bits, and 32-bit
+// adds to shared memory are one instruction where 64-bit ones are a loop around
+// compare-and-swap, whose lanes all meet at one chunk (a region's candidates are
+// neighbours). With those the cuts held rows of many candidates up: 64 requests
+// of 24,515 fp32 columns (Gaussian, sigma 2, top-p 0.9) took 117 us a step, 81
+// now, and 1024 of Zipf logits 1572 and 1495.
+struct MassSum {
+  uint32_t lo[kBuckets], hi[kBuckets];
+  __device__ __forceinline__ void clear(int i) { lo[i] = hi[i] = 0u; }
+  __device__ __forceinline__ void add(int i, unsigned long long m) {
+    atomicAdd(&lo[i], uint32_t(m) & 0xfffffu);
+    atomicAdd(&hi[i], uint32_t(m >> 20));
+  }
+  __device__ __forceinline__ unsigned long long get(int i) const {
+    return (static_cast<unsigned long long>(hi[i]) << 20) + lo[i];
+  }
+};
+static_assert(kSW * kRegion <= 4000, "the sums of a row fit 32 bits");
+
 struct NrSmem {
   char stage[kSW][kStage];
   NrRow r[2];
   union {  // the cut's phases, one after the other
-    unsigned long long mass[kBuckets];
+    MassSum mass;  // of the buckets
     struct {
       Cand gc[kCross];
       unsigned long long gm[kCross];
     } x;
-    unsigned long long cacc[kBuckets];
+    MassSum cacc;  // of the chunks
   } u;
   uint64_t full[kSW];          // the warp's unit has arrived
   uint64_t named[kQueue], taken[kQueue];  // the queue's entry is there / read by every warp
@@ -620,7 +640,7 @@ __device__ void cut_rows(const NucRowArgs& a, NrSmem& sm, int tid) {
       sm.n_gc = 0;
       sm.best = 0ull;
     }
-    for (int i = tid; i < kBuckets; i += kCT) sm.u.mass[i] = 0ull;
+    for (int i = tid; i < kBuckets; i += kCT) sm.u.mass.clear(i);
     cut_sync();
     if (!sm.ok || R.row < 0) return;
     const bool tgt = R.set != 0;
@@ -679,12 +699,12 @@ __device__ void cut_rows(const NucRowArgs& a, NrSmem& sm, int tid) {
     };
     bool settled = false;
     if (sound) {
-      for_cands([&](float z, int) { atomicAdd(&sm.u.mass[bucket(z)], fixm(z)); });
+      for_cands([&](float z, int) { sm.u.mass.add(bucket(z), fixm(z)); });
       cut_sync();
       const unsigned long long thr = sm.thr;
       // the bucket whose inclusive running mass reaches thr, and the mass before it
-      unsigned long long m0 = 2 * tid < kBuckets ? sm.u.mass[2 * tid] : 0ull;
-      unsigned long long m1 = 2 * tid + 1 < kBuckets ? sm.u.mass[2 * tid + 1] : 0ull;
+      unsigned long long m0 = 2 * tid < kBuckets ? sm.u.mass.get(2 * tid) : 0ull;
+      unsigned long long m1 = 2 * tid + 1 < kBuckets ? sm.u.mass.get(2 * tid + 1) : 0ull;
       unsigned long long incl = m0 + m1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -742,18 +762,18 @@ __device__ void cut_rows(const NucRowArgs& a, NrSmem& sm, int tid) {
           const float tau = sm.tau_v;
           const int tau_col = sm.tau_c;
           // the kept candidates join their chunks; the header
-          for (int c = tid; c < nch; c += kCT) sm.u.cacc[c] = 0ull;
+          for (int c = tid; c < nch; c += kCT) sm.u.cacc.clear(c);
           cut_sync();
           for_cands([&](float z, int x) {
-            if (z > tau || (z == tau && x <= tau_col)) atomicAdd(&sm.u.cacc[x / kChunk], fixm(z));
+            if (z > tau || (z == tau && x <= tau_col)) sm.u.cacc.add(x / kChunk, fixm(z));
           });
           cut_sync();
           unsigned long long tot = 0ull;  // whole numbers: the same in any order
-          for (int c = lane; c < nch; c += 32) tot += sm.u.cacc[c];
+          for (int c = lane; c < nch; c += 32) tot += sm.u.cacc.get(c);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
           const KeptNorm kn = kept_norm(tot);
-          for (int c = tid; c < nch; c += kCT) um[c] = kept_share(sm.u.cacc[c], kn);
+          for (int c = tid; c < nch; c += kCT) um[c] = kept_share(sm.u.cacc.get(c), kn);
           if (tid == 0) {
             const KeptScale ks = kept_scale(kn, M);
             *head = KeptHead{ks.lse, 1, tau, tau_col, M, ks.inv_s};
