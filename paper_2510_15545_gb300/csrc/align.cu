@@ -252,15 +252,44 @@ __device__ __forceinline__ int long_cost(const AlignArgs& a, const PairSmem& sm,
 }
 
 // The band's cells with a token of more than 8 bytes; a cost above kMaxCost is
-// stored as that and recomputed in the sweep.
+// stored as that and recomputed in the sweep. The cells lie scattered (a long
+// token's row and column), and the recurrence takes thousands of cycles: a warp
+// looks 32 cells over at a time and queues those it finds, one per lane, until
+// every lane has one. (With each cell computed where it was found, one or two
+// lanes worked at a time: 1024 pairs of 16 x 20 tokens, one in fifty long, took
+// 86 us; 40 now.)
 __device__ __noinline__ void long_costs(const AlignArgs& a, int d0, int t0, PairSmem sm,
                                         PairDims d, int t, int nt) {
-  for (int q = t; q < d.k * d.m; q += nt) {
-    const int i = q / d.m + 1, j = q - (i - 1) * d.m + 1, p = (i - 1) >> 1;
-    if (abs(i - j) > d.W0 || (sm.len_d[i - 1] <= 8 && sm.len_t[j - 1] <= 8)) continue;
+  const int lane = t & 31;
+  int held = 0, cell = 0;  // lanes below `held` have a cell queued
+  auto compute = [&]() {
+    const int i = cell / d.m + 1, j = cell - (i - 1) * d.m + 1, p = (i - 1) >> 1;
     sm.tile[16 * (p * d.nb - first_block(p, d.W0)) + 2 * (i + j - 2) + ((i - 1) & 1)] =
         uint8_t(min(long_cost(a, sm, d0, t0, i, j), kMaxCost));
+  };
+  for (int q0 = t - lane; q0 < d.k * d.m; q0 += nt) {
+    const int q = q0 + lane;
+    bool mine = q < d.k * d.m;
+    if (mine) {
+      const int i = q / d.m + 1, j = q - (i - 1) * d.m + 1;
+      mine = abs(i - j) <= d.W0 && (sm.len_d[i - 1] > 8 || sm.len_t[j - 1] > 8);
+    }
+    for (unsigned found = __ballot_sync(0xffffffffu, mine); found;) {
+      // lane held + x takes the x-th cell found
+      const int x = lane - held, n = __popc(found), take = min(32 - held, n);
+      const int src = x >= 0 && x < take ? int(__fns(found, 0, x + 1)) : 0;
+      const int c = __shfl_sync(0xffffffffu, q, src);
+      if (x >= 0 && x < take) cell = c;
+      held += take;
+      found = take == n ? 0u : found & ~((2u << __fns(found, 0, take)) - 1u);
+      if (held == 32) {
+        compute();
+        __syncwarp();
+        held = 0;
+      }
+    }
   }
+  if (lane < held) compute();
 }
 
 // One anti-diagonal of NP row pairs of a lane. cost: the pairs' entries of

@@ -16,7 +16,7 @@ from _parity import to_np
 pytestmark = pytest.mark.gpu
 
 
-def _check(ks, ms, max_len, symbols, windows, seed, n_vocab=200, min_len=0):
+def _check(ks, ms, max_len, symbols, windows, seed, n_vocab=200, min_len=0, n_long=0):
     if not torch.cuda.is_available():
         pytest.skip("needs a GPU")
     tt.load(build_if_missing=True)
@@ -25,6 +25,9 @@ def _check(ks, ms, max_len, symbols, windows, seed, n_vocab=200, min_len=0):
     while len(strings) < n_vocab:
         strings.add(bytes(rng.choice(symbols, size=int(rng.integers(min_len, max_len + 1)))
                           .astype(np.uint8)))
+    while len(strings) < n_vocab + n_long:  # some of 9 to 20 bytes
+        strings.add(bytes(rng.choice(symbols, size=int(rng.integers(9, 21))).astype(np.uint8)))
+    n_vocab = len(strings)
     voc = W.Vocab.from_strings(sorted(strings))
     d_off = np.concatenate([[0], np.cumsum(ks)]).astype(np.int32)
     t_off = np.concatenate([[0], np.cumsum(ms)]).astype(np.int32)
@@ -79,3 +82,14 @@ def test_costs_past_16_bits():
 
 def test_bands_wider_than_any_pair():
     _check([3, 64, 200], [5, 90, 300], 8, np.arange(97, 117), (767, 768, 2**30, 2**31 - 1), 9)
+
+
+@pytest.mark.parametrize("n_long", [1, 5, 30, 200])
+def test_a_few_long_tokens(n_long):
+    """Cells of long tokens scattered over the band, fewer and more than a warp
+    takes at once, on one warp, four warps and sixteen per pair."""
+    rng = np.random.default_rng(n_long)
+    args = (8, np.arange(97, 117), (0, 3, 8, -1), n_long)
+    _check(rng.integers(1, 20, size=60), rng.integers(1, 25, size=60), *args, n_long=n_long)
+    _check([64] * 400, rng.integers(40, 90, size=400), *args, n_long=n_long)
+    _check([200, 130, 64], [250, 31, 90], *args, n_long=n_long)
