@@ -257,11 +257,12 @@ def default_steps(name: str) -> int:
             "dtw_4096x64": 1000, "b1024_g8_v201k_bf16": 1000}.get(name, 1000)
 
 
-def step_launches(args) -> int:
+def step_launches(args, batch: int = 0) -> int:
     """Kernels one tt_step launches: alignment, row pass and decision; with
     filters also the kept sets of top-k families, the nucleus kernel of
     top-p-only families and the transfer of q_hat before the decision."""
-    pen = 1 if args.rep_penalty != 1.0 else 0  # the penalty's per-request sets
+    # the penalty's per-request sets, and the look over the offsets of large batches
+    pen = (2 if batch > 1024 else 1) if args.rep_penalty != 1.0 else 0
     if args.top_k > 0:
         return 5 + pen
     if args.top_p < 1.0:
@@ -617,7 +618,7 @@ def run_mine(args):
                      "peak_kind": "%s copy bandwidth (hbm_gbs)" % peak_kind,
                      "traffic": traffic, "algorithmic_bytes": ab["total"],
                      "vs_nominal_8tbs": achieved / 8000.0},
-        "gpu_launches": step_launches(args) * K,
+        "gpu_launches": step_launches(args, wl.B) * K,
         "clocks": clk,
     }
     if e2e is not None:

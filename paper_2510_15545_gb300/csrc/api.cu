@@ -151,6 +151,7 @@ cudaError_t launch_pen_sets(const tt_batch* batch, const RowSet& d, const RowSet
   a.pcnt_t = ws.pcnt_t;
   a.pstart_t = ws.pstart_t;
   a.pstatus = ws.pstatus;
+  a.fell = ws.fell;
   return launch_pen_prep(a, s);
 }
 

@@ -85,6 +85,7 @@ struct Workspace {
   int32_t* status;   // [B] per-request status between kernels
   int32_t* excl;     // [n_target + B] scored column of each target row (-1: bonus row)
   int32_t* err;      // two words: epoch of a call whose row pass failed, and why
+  int32_t* fell;     // two words of the penalty's sets (see PenArgs), behind err
   unsigned long long* work;  // row-pass work counters (kWorkShards, kWorkStride apart), zeroed
                              // by the kernel before the row pass
   Cand* cand_d;      // [n_draft * nch_d * cand_stride(k_d)] top-k lists of filtered draft rows
@@ -133,7 +134,8 @@ __host__ __device__ inline Workspace workspace_layout(void* base, int B, int n_d
   w.q_hat = reinterpret_cast<float*>(take(sizeof(float) * size_t(n_target)));
   w.status = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * size_t(B)));
   w.excl = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * rows_t));
-  w.err = reinterpret_cast<int32_t*>(take(2 * sizeof(int32_t)));
+  w.err = reinterpret_cast<int32_t*>(take(4 * sizeof(int32_t)));
+  w.fell = w.err ? w.err + 2 : nullptr;
   w.work = reinterpret_cast<unsigned long long*>(take(kWorkShards * kWorkStride * sizeof(unsigned long long)));
   w.cand_d = reinterpret_cast<Cand*>(
       take(sizeof(Cand) * size_t(n_draft) * n_chunks(V_d) * size_t(k_d > 0 ? cand_stride(k_d) : 0)));

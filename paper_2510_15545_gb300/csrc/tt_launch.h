@@ -230,6 +230,7 @@ struct PenArgs {
   int32_t* pcnt_t;
   int32_t* pstart_t;
   int32_t* pstatus;
+  int32_t* fell;  // two words of scratch: whether a family's offsets fall anywhere
 };
 
 struct PrepArgs {

@@ -171,6 +171,7 @@ def test_launch_count_traffic_and_filters_key_follow_the_run_filters():
     assert bench.step_launches(p(["--top-k", "20", "--top-p", "0.95"])) == 5
     assert bench.step_launches(p(["--top-p", "0.9"])) == 6
     assert bench.step_launches(p(["--top-k", "20", "--rep-penalty", "1.1"])) == 6
+    assert bench.step_launches(p(["--top-k", "20", "--rep-penalty", "1.1"]), 4096) == 7
     assert bench.run_traffic("no_such_workload", p(["--top-p", "0.9"])) is None
     assert bench.run_traffic("no_such_workload",
                              p(["--top-k", "20", "--rep-penalty", "1.1"])) is None

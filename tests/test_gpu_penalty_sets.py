@@ -87,6 +87,35 @@ def _with_offsets(wl, off):
                                hist_off_d=np.array(off, np.int32))
 
 
+@pytest.mark.parametrize("B", [1024, 1025, 3000])
+def test_bad_history_ranges_in_large_batches(B):
+    """The two ways the offsets are looked over (by every CTA, and by a kernel
+    ahead of them from 1025 requests on): falls at both ends of the batch."""
+    G, V, L = 2, 300, 30
+    wl = W.homogeneous_workload(B, G, V, seed=B, logit_scale=2.0)
+    rng = np.random.default_rng(B)
+    good = np.arange(B + 1) * L
+    off = good.copy()
+    off[2] = off[1] - 5      # request 1 is bad; request 2 reaches back 35: into request 0's place
+    off[B - 1] = off[B] + 7  # request B - 2 takes more than its share, B - 1 is bad
+    cols = rng.integers(0, V, size=B * L + 7).astype(np.int32)
+    wl = dataclasses.replace(wl, hist_cols_t=cols, hist_cols_d=cols)
+    inp = tt.device_inputs(_with_offsets(wl, off), "cuda")
+    inp["batch"].n_hist_d = inp["batch"].n_hist_t = B * L + 7
+    for k, v in PEN.items():
+        setattr(inp["params"], k, v)
+    g = to_np(tt.tt_step(inp["batch"], inp["vd"], inp["vt"], _padded(wl.draft_logits),
+                         _padded(wl.target_logits), inp["params"]))
+    bad = [1, 2, B - 1]
+    assert np.all(g["status"][bad] == oracle.ST_BAD_OFFSETS)
+    assert np.all(np.delete(g["status"], bad) == 0)
+    g["_target_off"], g["_draft_off"] = wl.target_off, wl.draft_off
+    whole = _with_offsets(wl, off)
+    for b in [0, 3, B // 2, B - 3, B - 2]:
+        sw = whole.subset([b])
+        compare(sw, dict(g), oracle_step(sw, request_base=b, **PEN), req_index=[b])
+
+
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("bad,refused,off", [
     # which request's range is bad, which others are refused, the offset after it
