@@ -396,7 +396,7 @@ __device__ bool candidate_cut(double Td, NucSmem& sm, const char* row, int dt, i
     const float f = __fsub_rn(M, __fmul_rn(z, scale)) * kBucketsPerUnit;
     return f > 0.f ? min(kCandBuckets - 1, int(f)) : 0;
   };
-  for_cands([&](const Cand& e) { atomicAdd(&sm.mass[bucket(e.v)], fixm(e.v)); });
+  for_cands([&](const Cand& e) { shared_add_u64(&sm.mass[bucket(e.v)], fixm(e.v)); });
   __syncthreads();
   // the first bucket whose inclusive running mass reaches thr (thread t owns a
   // contiguous run of buckets)
@@ -478,7 +478,8 @@ __device__ bool candidate_cut(double Td, NucSmem& sm, const char* row, int dt, i
   }
   // the kept candidates join their chunks
   for_cands([&](const Cand& e) {
-    if (e.v > tau || (e.v == tau && e.c <= tau_col)) atomicAdd(&sm.cacc[e.c / kChunk], fixm(e.v));
+    if (e.v > tau || (e.v == tau && e.c <= tau_col))
+      shared_add_u64(&sm.cacc[e.c / kChunk], fixm(e.v));
   });
   return ng > 0;
 }
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
     }
     for (int i = lane; i < n; i += 32) {
       const Cand e = sm.cand[i];
-      atomicAdd(&sm.mass[bucket(e.v)], fixm(e.v));
+      shared_add_u64(&sm.mass[bucket(e.v)], fixm(e.v));
     }
     __syncwarp();
     // the first bucket whose inclusive running mass reaches thr (lane l owns a
@@ -665,7 +666,7 @@ __global__ void __launch_bounds__(kWWarps * 32, 3) nucleus_warp_kernel(KeptArgs 
     for (int i = lane; i < n; i += 32) {
       const Cand c = sm.cand[i];
       if (c.v > tau || (c.v == tau && c.c <= tau_col))
-        atomicAdd(&sm.cacc[c.c / kChunk], fixm(c.v));
+        shared_add_u64(&sm.cacc[c.c / kChunk], fixm(c.v));
     }
     __syncwarp();
     unsigned long long tot = lane < nch ? sm.cacc[lane] : 0ull;
@@ -818,7 +819,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
         if (p.b[0] < 0) return;
         if (level > 0 && path_cmp(p, cross, level - 1) != 0) return;
         atomicAdd(&sm.cnt[p.b[level]], 1u);
-        atomicAdd(&sm.mass[p.b[level]], fixm(z));
+        shared_add_u64(&sm.mass[p.b[level]], fixm(z));
       });
       __syncthreads();
       // running mass over the buckets (thread t owns a contiguous run of them)
@@ -882,7 +883,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
       if (p.b[0] < 0) return;
       const int c = all_kept ? -1 : path_cmp(p, cross, level);
       if (c < 0) {
-        atomicAdd(&sm.cacc[x / kChunk], fixm(z));
+        shared_add_u64(&sm.cacc[x / kChunk], fixm(z));
       } else if (c == 0) {
         const int i = atomicAdd(&sm.n_gz, 1);
         if (i < kGather) sm.gz[i] = Cand{z, x};
@@ -897,7 +898,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
         for (int i = tid; i < ng; i += kNT) {
           const Cand e = sm.gz[i];
           if (e.v > tau || (e.v == tau && e.c <= tau_col))
-            atomicAdd(&sm.cacc[e.c / kChunk], fixm(e.v));
+            shared_add_u64(&sm.cacc[e.c / kChunk], fixm(e.v));
         }
       } else {
         // a crossing run of more than kGather tied columns (the last level holds
@@ -968,7 +969,7 @@ __global__ void __launch_bounds__(kNT, 3) nucleus_kernel(KeptArgs a) {
           const Path p = bucket_path(d);
           if (p.b[0] >= 0 && path_cmp(p, cross, level) == 0 &&
               (z > tau || (z == tau && x <= tau_col)))
-            atomicAdd(&sm.cacc[x / kChunk], fixm(z));
+            shared_add_u64(&sm.cacc[x / kChunk], fixm(z));
         });
       }
     }

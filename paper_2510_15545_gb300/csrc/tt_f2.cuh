@@ -54,6 +54,19 @@ __device__ __forceinline__ float exp2_scaled(float z, float scale, float M) {
   return ex2_approx(f) * __int_as_float((int(n) + 127) << 23);
 }
 
+// Adds m to a 64-bit sum in shared memory by 32-bit adds, the carry from the lower
+// word's old value (the sum is whole once all adds are done: read it past a
+// barrier). A 64-bit atomicAdd is a loop around compare-and-swap there, and lanes
+// that meet at one sum, as the candidates of a region do at one chunk, go round
+// it in turn: 64 requests of 151,936 fp32 columns whose rows need the histogram
+// levels (Gaussian logits, sigma 1, top-p 0.9) take 1562 us a step, 2792 with it.
+__device__ __forceinline__ void shared_add_u64(unsigned long long* sum, unsigned long long m) {
+  unsigned int* w = reinterpret_cast<unsigned int*>(sum);
+  const unsigned int lo = static_cast<unsigned int>(m), old = atomicAdd(w, lo);
+  const unsigned int hi = static_cast<unsigned int>(m >> 32) + (old + lo < old ? 1u : 0u);
+  if (hi) atomicAdd(w + 1, hi);
+}
+
 // The kept set of a nucleus row from its kept mass `tot` (40-bit fixed point,
 // relative to 2^M). Every kernel that settles nucleus rows forms these the same
 // way, so that a row's result does not depend on which did.
