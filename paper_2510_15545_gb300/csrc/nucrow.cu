@@ -334,8 +334,9 @@ __device__ __forceinline__ uint32_t vec_max_bf16(const uint4& w) {
 // where it stands and by whole log2 units, until the unit's vectors that reach it
 // (a candidate each, at least) leave room. From 14 down in each unit, with a
 // gathering after each step, it held flat rows up: 64 requests of Gaussian
-// logits (sigma 1.5, fp32, 151,936 columns, top-p 0.9) took 2281 us, 2061 now;
-// the two kernels that this one replaced, 1954.
+// logits (sigma 1.5, fp32, 151,936 columns, top-p 0.9) took 2281 us, so 2061
+// (1663 with the sums by 32-bit adds; the two kernels that this one replaced
+// took 1950).
 struct NrBar {
   float bar, zc;
   uint32_t flags;  // the vectors that reach it

@@ -49,11 +49,11 @@ constexpr int kNucWideRows = 2;
 // stay unused. Against the row pass and the kernels after it, on Zipf logits
 // (both families of one width):
 //                        64 requests, top-p 0.95   512 requests, top-p 0.9
-//   bf16 10,000 (2.4 units)    115 us to 89             490 us to 441
-//   bf16 16,323 (4.0)          102 us to 97             447 us to 509
-//   bf16 20,419 (5.0)           98 us to 103            430 us to 580
-//   fp32  9,155 (4.5)           95 us to 96             409 us to 500
-//   fp32 16,323 (8.0)           92 us to 105            396 us to 569
+//   bf16 10,000 (2.4 units)     94 us to 79             411 us to 392
+//   bf16 16,323 (4.0)           88 us to 87             394 us to 459
+//   bf16 20,419 (5.0)           84 us to 94             387 us to 509
+//   fp32  9,155 (4.5)           80 us to 87             371 us to 456
+//   fp32 16,323 (8.0)           80 us to 98             367 us to 527
 constexpr int kNucRowUnits = 4;
 constexpr int kNucWideMax = 480 * 2048;
 inline int nucleus_rows(bool nucleus, int V, int unit_cols) {
